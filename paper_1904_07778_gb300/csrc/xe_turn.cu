@@ -37,6 +37,36 @@ __device__ __forceinline__ void st32B(uint8_t* p, const uint32_t (&r)[8]) {
                : "memory");
 }
 
+// 16 bytes from any address: the two aligned 16-byte words around it (one if
+// it is aligned) and a byte shift.  A word that reaches outside [begin, end)
+// is not read: its bytes come one by one, and those outside are zero.
+__device__ __forceinline__ void ld16_any(const uint8_t* p, const uint8_t* begin, const uint8_t* end,
+                                         uint32_t (&r)[4]) {
+  const uint32_t a = (uint32_t)(reinterpret_cast<uintptr_t>(p) & 15);
+  const uint8_t* q = p - a;
+  if (q >= begin && q + (a ? 32 : 16) <= end) {
+    const uint4 lo = __ldg(reinterpret_cast<const uint4*>(q));
+    uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, 0u, 0u, 0u, 0u};
+    if (a) {
+      const uint4 hi = __ldg(reinterpret_cast<const uint4*>(q + 16));
+      w[4] = hi.x, w[5] = hi.y, w[6] = hi.z, w[7] = hi.w;
+    }
+#pragma unroll
+    for (int i = 0; i < 6; ++i) w[i] = (a & 8) ? w[i + 2] : w[i];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) w[i] = (a & 4) ? w[i + 1] : w[i];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) r[i] = __funnelshift_r(w[i], w[i + 1], 8 * (a & 3));
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      r[i] = 0;
+      for (int b = 0; b < 4; ++b)
+        if (p + 4 * i + b >= begin && p + 4 * i + b < end) r[i] |= (uint32_t)p[4 * i + b] << (8 * b);
+    }
+  }
+}
+
 __device__ __forceinline__ int tile_word(int row, int w) { return row * 32 + (w ^ ((row >> 5) << 2)); }
 
 // barrier of one 256-thread group (id 0 is the whole CTA of a 256-thread launch)
@@ -45,10 +75,11 @@ __device__ __forceinline__ void group_bar(int id) {
 }
 
 // Store phase of a tile held in `tile`: each thread transposes 4 x 32 bytes
-// in registers and writes 32-byte pieces of [k][g][t] rows.
+// in registers and writes 32-byte pieces of [k][g][t] rows (vec: the rows are
+// aligned to and padded to 32 bytes), or single bytes.
 __device__ __forceinline__ void turn_tile_store(uint8_t* __restrict__ out, int T, int K, int G,
                                                 long long os, int pair_rows, int t0, int k0,
-                                                int g, const uint32_t* tile, int tid, bool full) {
+                                                int g, const uint32_t* tile, int tid, bool full, bool vec) {
   const int warp = tid >> 5, lane = tid & 31;
   // store: thread = 4 consecutive k (word kq) x 32 consecutive t (segment ts);
   // the eight lanes of a k-quad cover one 256-byte stretch of each output row
@@ -66,11 +97,11 @@ __device__ __forceinline__ void turn_tile_store(uint8_t* __restrict__ out, int T
     const long long row =
         pair_rows ? ((long long)(k >> 1) * G + g) * 2 + (k & 1) : (long long)k * G + g;
     uint8_t* o = out + row * os + tb;
-    if (full) {
+    if (full || (vec && k < K && tb < T)) {  // the last piece of a row runs into its padding (zeros)
       const uint32_t r[8] = {a[c], a[4 + c], a[8 + c], a[12 + c],
                              a[16 + c], a[20 + c], a[24 + c], a[28 + c]};
       st32B(o, r);
-    } else if (k < K) {
+    } else if (!vec && k < K) {
       for (int b = 0; b < 32; ++b)
         if (tb + b < T) o[b] = (uint8_t)(a[4 * (b >> 2) + c] >> ((b & 3) * 8));
     }
@@ -78,17 +109,40 @@ __device__ __forceinline__ void turn_tile_store(uint8_t* __restrict__ out, int T
 }
 
 
+// Which accesses of a turn may be 32 bytes wide.
+enum : int { kTurnIn = 1, kTurnOut = 2 };
+
+// Load of a tile at an edge, or of unaligned rows: 16-byte pieces from any
+// address, zeros past K and T.  Not inlined: its registers stay out of the
+// kernels' main path.
+__device__ __noinline__ void turn_tile_edge_load(const uint8_t* __restrict__ in, int T, int G, int K,
+                                                 long long ks, int t0, int k0, int g, uint32_t* tile,
+                                                 int tid) {
+  const uint8_t* const end = in + ((long long)T * G - 1) * ks + K;
+#pragma unroll 4
+  for (int it = 0; it < 8; ++it) {
+    const int e = it * 256 + tid, r = e >> 3, c = e & 7;
+    uint32_t x[4] = {0u, 0u, 0u, 0u};
+    if (t0 + r < T && k0 + 16 * c < K)
+      ld16_any(in + ((long long)(t0 + r) * G + g) * ks + k0 + 16 * c, in, end, x);
+    *reinterpret_cast<uint4*>(&tile[tile_word(r, 4 * c)]) = make_uint4(x[0], x[1], x[2], x[3]);
+  }
+}
+
 // One tile: 256 threads (tid 0..255) move spectra t0 .. t0+255 of byte rows
 // k0 .. k0+127 of group g through `tile`, meeting at barrier `bar`.  Input
 // row (t, g) starts at in + (t G + g) ks: ks = K, or more for a range of
-// rows cut from a wider block.
+// rows cut from a wider block.  Tiles at the edges, and every tile of a block
+// whose rows are not 32-byte aligned, load through ld16_any (HBM-bound as
+// the aligned ones: a 100-input, 333-channel, 3001-spectra block, pushed and
+// dumped, takes 0.132 ms, against 0.630 ms with byte loads and stores).
 __device__ __forceinline__ void turn_tile(const uint8_t* __restrict__ in, uint8_t* __restrict__ out,
-                                          int T, int G, int K, long long ks, long long os, int vec_ok,
+                                          int T, int G, int K, long long ks, long long os, int vec,
                                           int pair_rows, int t0, int k0, int g, uint32_t* tile,
                                           int tid, int bar) {
-  const bool full = vec_ok && t0 + kTT <= T && k0 + kTK <= K;
   // load: 256 rows x 128 bytes as 32-byte pieces, four per thread, all
   // issued before any of them is stored
+  const bool full = vec == (kTurnIn | kTurnOut) && t0 + kTT <= T && k0 + kTK <= K;
   if (full) {
     uint32_t v[4][8];
 #pragma unroll
@@ -108,27 +162,18 @@ __device__ __forceinline__ void turn_tile(const uint8_t* __restrict__ in, uint8_
       *reinterpret_cast<uint4*>(&tile[tile_word(r, 8 * p + (odd ? 0 : 4))]) = odd ? lo : hi;
     }
   } else {
-    for (int e = tid; e < kTT * 32; e += 256) {
-      const int r = e >> 5, w = e & 31;
-      uint32_t x = 0;
-      if (t0 + r < T) {
-        const long long off = ((long long)(t0 + r) * G + g) * ks + k0 + 4 * w;
-        for (int b = 0; b < 4; ++b)
-          if (k0 + 4 * w + b < K) x |= (uint32_t)in[off + b] << (8 * b);
-      }
-      tile[tile_word(r, w)] = x;
-    }
+    turn_tile_edge_load(in, T, G, K, ks, t0, k0, g, tile, tid);
   }
   group_bar(bar);
-  turn_tile_store(out, T, K, G, os, pair_rows, t0, k0, g, tile, tid, full);
+  turn_tile_store(out, T, K, G, os, pair_rows, t0, k0, g, tile, tid, full, (vec & kTurnOut) != 0);
 }
 
 __global__ void __launch_bounds__(256, 4) turn_kernel(const uint8_t* __restrict__ in,
                                                       uint8_t* __restrict__ out, int T, int G,
                                                       int K, long long ks, long long os,
-                                                      int vec_ok, int pair_rows) {
+                                                      int vec, int pair_rows) {
   __shared__ __align__(16) uint32_t tile[kTT * 32];
-  turn_tile(in, out, T, G, K, ks, os, vec_ok, pair_rows, blockIdx.x * kTT, blockIdx.y * kTK,
+  turn_tile(in, out, T, G, K, ks, os, vec, pair_rows, blockIdx.x * kTT, blockIdx.y * kTK,
             blockIdx.z, tile, threadIdx.x, 0);
 }
 
@@ -138,7 +183,7 @@ __global__ void __launch_bounds__(256, 4) turn_kernel(const uint8_t* __restrict_
 // keeps in flight, not by HBM: each of the kTurnGroups 256-thread groups of a
 // CTA walks its own tiles through kTurnBufs 32 KB buffers, with the 16-byte
 // cp.async copies of the next kTurnBufs - 1 tiles in flight while one tile is
-// transposed and stored.  Edge tiles take the byte path synchronously.
+// transposed and stored.  Edge tiles load synchronously.
 #ifndef XE_TURN_GROUPS
 #define XE_TURN_GROUPS 3
 #endif
@@ -179,7 +224,7 @@ __device__ __forceinline__ void tile_prefetch(const uint8_t* __restrict__ in, in
 
 __global__ void __launch_bounds__(256 * kTurnGroups, 1)
     turn_persist_kernel(const uint8_t* __restrict__ in, uint8_t* __restrict__ out, int T, int G,
-                        int K, long long ks, long long os, int vec_ok, int pair_rows) {
+                        int K, long long ks, long long os, int vec, int pair_rows) {
   extern __shared__ __align__(16) uint32_t tiles[];
   const int grp = threadIdx.x >> 8, tid = threadIdx.x & 255, bar = 1 + grp;
   uint32_t* const mine = tiles + kTurnBufs * grp * kTileWords;  // this group's buffers
@@ -194,7 +239,7 @@ __global__ void __launch_bounds__(256 * kTurnGroups, 1)
     k0 = (int)(r - q * gy) * kTK;
     g = (int)q;
   };
-  auto is_full = [&](int t0, int k0) { return vec_ok && t0 + kTT <= T && k0 + kTK <= K; };
+  auto is_full = [&](int t0, int k0) { return vec == (kTurnIn | kTurnOut) && t0 + kTT <= T && k0 + kTK <= K; };
   // copies of full tile w into buffer b; one commit group per tile, empty
   // for edge tiles and past the end, so that group i is always tile i
   auto prefetch = [&](unsigned w, int b) {
@@ -219,9 +264,9 @@ __global__ void __launch_bounds__(256 * kTurnGroups, 1)
     uint32_t* tile = mine + b * kTileWords;
     if (is_full(t0, k0)) {
       group_bar(bar);
-      turn_tile_store(out, T, K, G, os, pair_rows, t0, k0, g, tile, tid, true);
+      turn_tile_store(out, T, K, G, os, pair_rows, t0, k0, g, tile, tid, true, true);
     } else {
-      turn_tile(in, out, T, G, K, ks, os, vec_ok, pair_rows, t0, k0, g, tile, tid, bar);
+      turn_tile(in, out, T, G, K, ks, os, vec, pair_rows, t0, k0, g, tile, tid, bar);
     }
     group_bar(bar);
     if (++b == kTurnBufs) b = 0;
@@ -240,8 +285,24 @@ __global__ void __launch_bounds__(256 * kTurnGroups, 1)
 struct PktGeom {
   int n_fids, inputs_pkt, n_xids, chans_pkt, T;
   long long os;
-  int vec_ok;
+  int vec_in;   // 32-byte aligned packet rows
+  int width;    // widest store every output row's 32-byte pieces allow: 32, 16, 8 or 1 byte(s)
 };
+
+__device__ __noinline__ void pkt_tile_edge_load(const uint8_t* __restrict__ in,
+                                                const uint8_t* __restrict__ base, int T, int rowb,
+                                                long long slot_stride, int t0, int k0, uint32_t* tile,
+                                                int tid) {
+  const uint8_t* const end = in + (long long)(T >> 3) * slot_stride;
+#pragma unroll 4
+  for (int it = 0; it < 8; ++it) {
+    const int e = it * 256 + tid, r = e >> 3, c = e & 7, t = t0 + r;
+    uint32_t x[4] = {0u, 0u, 0u, 0u};
+    if (t < T && k0 + 16 * c < rowb)
+      ld16_any(base + (long long)(t >> 3) * slot_stride + (long long)(t & 7) * rowb + k0 + 16 * c, in, end, x);
+    *reinterpret_cast<uint4*>(&tile[tile_word(r, 4 * c)]) = make_uint4(x[0], x[1], x[2], x[3]);
+  }
+}
 
 __global__ void __launch_bounds__(256, 4) pkt_turn_kernel(const uint8_t* __restrict__ in,
                                                           uint8_t* __restrict__ out, PktGeom q) {
@@ -254,7 +315,7 @@ __global__ void __launch_bounds__(256, 4) pkt_turn_kernel(const uint8_t* __restr
   const int N = q.n_fids * q.inputs_pkt;
   const uint8_t* base = in + ((long long)fid * q.n_xids + xid) * P;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const bool full = q.vec_ok && t0 + kTT <= q.T && k0 + kTK <= rowb;
+  const bool full = q.vec_in && t0 + kTT <= q.T && k0 + kTK <= rowb;
   if (full) {
     uint32_t v[4][8];
 #pragma unroll
@@ -272,16 +333,7 @@ __global__ void __launch_bounds__(256, 4) pkt_turn_kernel(const uint8_t* __restr
       *reinterpret_cast<uint4*>(&tile[tile_word(r, 8 * p + (odd ? 0 : 4))]) = odd ? lo : hi;
     }
   } else {
-    for (int e = tid; e < kTT * 32; e += 256) {
-      const int r = e >> 5, w = e & 31, t = t0 + r;
-      uint32_t x = 0;
-      if (t < q.T) {
-        const uint8_t* src = base + (long long)(t >> 3) * slot_stride + (long long)(t & 7) * rowb;
-        for (int b = 0; b < 4; ++b)
-          if (k0 + 4 * w + b < rowb) x |= (uint32_t)src[k0 + 4 * w + b] << (8 * b);
-      }
-      tile[tile_word(r, w)] = x;
-    }
+    pkt_tile_edge_load(in, base, q.T, rowb, slot_stride, t0, k0, tile, tid);
   }
   __syncthreads();
   const int kq = 4 * warp + (lane >> 3), ts = lane & 7;
@@ -297,22 +349,37 @@ __global__ void __launch_bounds__(256, 4) pkt_turn_kernel(const uint8_t* __restr
     const int ch = xid * q.chans_pkt + k / q.inputs_pkt, inp = fid * q.inputs_pkt + k % q.inputs_pkt;
     const int tb = t0 + ts * 32;
     uint8_t* o = out + ((long long)ch * N + inp) * q.os + tb;
-    if (full) {
-      const uint32_t r[8] = {a[c], a[4 + c], a[8 + c], a[12 + c],
-                             a[16 + c], a[20 + c], a[24 + c], a[28 + c]};
+    const uint32_t r[8] = {a[c], a[4 + c], a[8 + c], a[12 + c],
+                           a[16 + c], a[20 + c], a[24 + c], a[28 + c]};
+    if (full && q.width == 32) {
       st32B(o, r);
+      continue;
+    }
+    const int n = q.T - tb;  // spectra left of the row: a multiple of 8
+    if (n <= 0) continue;
+    if (q.width == 32 && n >= 32) {
+      st32B(o, r);
+    } else if (q.width >= 16 && n >= 32) {
+      *reinterpret_cast<uint4*>(o) = make_uint4(r[0], r[1], r[2], r[3]);
+      *reinterpret_cast<uint4*>(o + 16) = make_uint4(r[4], r[5], r[6], r[7]);
+    } else if (q.width >= 8) {
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+        if (8 * b < n) *reinterpret_cast<uint2*>(o + 8 * b) = make_uint2(r[2 * b], r[2 * b + 1]);
     } else {
+#pragma unroll
       for (int b = 0; b < 32; ++b)
-        if (tb + b < q.T) o[b] = (uint8_t)(a[4 * (b >> 2) + c] >> ((b & 3) * 8));
+        if (b < n) o[b] = (uint8_t)(r[b >> 2] >> ((b & 3) * 8));
     }
   }
 }
 
 // ---------------------------------------------------------------- plane split
-// out[r][p][t] = in[r][t][p] for 8-bit complex samples: 16 samples (32 bytes)
-// per thread become 16 real and 16 imaginary bytes.
+// out[r][p][t] = in[r][t][p] for 8-bit complex samples: 16 samples (32 bytes,
+// any alignment) per thread become 16 real and 16 imaginary bytes.  The last
+// 16 of a row run into its padding (vec: rows aligned to and padded to 16).
 __global__ void split_planes_kernel(const uint8_t* __restrict__ in, uint8_t* __restrict__ out,
-                                    long long rows, int T, long long os, int vec_ok) {
+                                    long long rows, int T, long long os, int vec) {
   const int per_row = (T + 15) / 16;
   const long long total = rows * per_row;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
@@ -322,16 +389,17 @@ __global__ void split_planes_kernel(const uint8_t* __restrict__ in, uint8_t* __r
     const uint8_t* src = in + (r * T + t) * 2;
     uint8_t* dre = out + (2 * r) * os + t;
     uint8_t* dim = dre + os;
-    if (vec_ok && t + 16 <= T) {
-      const uint4 a = *reinterpret_cast<const uint4*>(src);
-      const uint4 b = *reinterpret_cast<const uint4*>(src + 16);
+    if (vec) {
+      uint32_t a[4], b[4];
+      ld16_any(src, in, in + rows * T * 2, a);
+      ld16_any(src + 16, in, in + rows * T * 2, b);
       // even bytes are real parts, odd bytes imaginary parts
       *reinterpret_cast<uint4*>(dre) =
-          make_uint4(__byte_perm(a.x, a.y, 0x6420), __byte_perm(a.z, a.w, 0x6420),
-                     __byte_perm(b.x, b.y, 0x6420), __byte_perm(b.z, b.w, 0x6420));
+          make_uint4(__byte_perm(a[0], a[1], 0x6420), __byte_perm(a[2], a[3], 0x6420),
+                     __byte_perm(b[0], b[1], 0x6420), __byte_perm(b[2], b[3], 0x6420));
       *reinterpret_cast<uint4*>(dim) =
-          make_uint4(__byte_perm(a.x, a.y, 0x7531), __byte_perm(a.z, a.w, 0x7531),
-                     __byte_perm(b.x, b.y, 0x7531), __byte_perm(b.z, b.w, 0x7531));
+          make_uint4(__byte_perm(a[0], a[1], 0x7531), __byte_perm(a[2], a[3], 0x7531),
+                     __byte_perm(b[0], b[1], 0x7531), __byte_perm(b[2], b[3], 0x7531));
     } else {
       for (int k = 0; k < 16 && t + k < T; ++k) {
         dre[k] = src[2 * k];
@@ -443,9 +511,9 @@ cudaError_t turn_launch_strided(const uint8_t* in, uint8_t* out, int T, int G, i
                                 long long in_stride, long long out_stride, cudaStream_t s,
                                 bool pair_rows, int persist_ctas) {
   if (in_stride < K) return cudaErrorInvalidValue;
-  const int vec_ok = (K % 32 == 0) && (in_stride % 32 == 0) && (T % 32 == 0) && (out_stride % 32 == 0) &&
-                     (reinterpret_cast<uintptr_t>(in) % 32 == 0) &&
-                     (reinterpret_cast<uintptr_t>(out) % 32 == 0);
+  const int vec =
+      (in_stride % 32 == 0 && reinterpret_cast<uintptr_t>(in) % 32 == 0 ? kTurnIn : 0) |
+      (out_stride % 32 == 0 && reinterpret_cast<uintptr_t>(out) % 32 == 0 ? kTurnOut : 0);
   const long long n_tiles = (long long)((T + kTT - 1) / kTT) * ((K + kTK - 1) / kTK) * G;
   if (persist_ctas > 0 && n_tiles + (long long)persist_ctas * kTurnGroups * kTurnBufs < (1LL << 31)) {
     constexpr int smem = kTurnGroups * kTurnBufs * kTileWords * (int)sizeof(uint32_t);
@@ -457,33 +525,32 @@ cudaError_t turn_launch_strided(const uint8_t* in, uint8_t* out, int T, int G, i
       attr = true;
     }
     turn_persist_kernel<<<persist_ctas, 256 * kTurnGroups, smem, s>>>(
-        in, out, T, G, K, in_stride, out_stride, vec_ok, pair_rows ? 1 : 0);
+        in, out, T, G, K, in_stride, out_stride, vec, pair_rows ? 1 : 0);
     return cudaGetLastError();
   }
   dim3 grid((T + kTT - 1) / kTT, (K + kTK - 1) / kTK, G);
-  turn_kernel<<<grid, 256, 0, s>>>(in, out, T, G, K, in_stride, out_stride, vec_ok, pair_rows ? 1 : 0);
+  turn_kernel<<<grid, 256, 0, s>>>(in, out, T, G, K, in_stride, out_stride, vec, pair_rows ? 1 : 0);
   return cudaGetLastError();
 }
 
 cudaError_t split_planes_launch(const uint8_t* in, uint8_t* out, long long rows, int T,
                                 long long out_stride, cudaStream_t s) {
-  const int vec_ok = (T % 16 == 0) && (out_stride % 16 == 0) &&
-                     (reinterpret_cast<uintptr_t>(in) % 16 == 0) &&
-                     (reinterpret_cast<uintptr_t>(out) % 16 == 0);
+  const int vec = out_stride % 16 == 0 && reinterpret_cast<uintptr_t>(out) % 16 == 0;
   const long long total = rows * ((T + 15) / 16);
   long long blocks = (total + 255) / 256;
   if (blocks > 152 * 16) blocks = 152 * 16;
   if (blocks < 1) blocks = 1;
-  split_planes_kernel<<<(unsigned)blocks, 256, 0, s>>>(in, out, rows, T, out_stride, vec_ok);
+  split_planes_kernel<<<(unsigned)blocks, 256, 0, s>>>(in, out, rows, T, out_stride, vec);
   return cudaGetLastError();
 }
 
 cudaError_t pkt_turn_launch(const uint8_t* in, uint8_t* out, int n_fids, int inputs_pkt, int n_xids,
                             int chans_pkt, int T, long long out_stride, cudaStream_t s) {
-  PktGeom q{n_fids, inputs_pkt, n_xids, chans_pkt, T, out_stride, 0};
+  PktGeom q{n_fids, inputs_pkt, n_xids, chans_pkt, T, out_stride, 0, 1};
   const int rowb = chans_pkt * inputs_pkt;
-  q.vec_ok = rowb % 32 == 0 && out_stride % 32 == 0 && T % 32 == 0 &&
-             reinterpret_cast<uintptr_t>(in) % 32 == 0 && reinterpret_cast<uintptr_t>(out) % 32 == 0;
+  q.vec_in = rowb % 32 == 0 && reinterpret_cast<uintptr_t>(in) % 32 == 0;
+  for (int w : {8, 16, 32})
+    if (out_stride % w == 0 && reinterpret_cast<uintptr_t>(out) % w == 0) q.width = w;
   dim3 grid((T + kTT - 1) / kTT, (rowb + kTK - 1) / kTK, n_fids * n_xids);
   pkt_turn_kernel<<<grid, 256, 0, s>>>(in, out, q);
   return cudaGetLastError();
