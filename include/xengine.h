@@ -277,7 +277,7 @@ typedef struct corr_stats {
   uint64_t blocks;          /* blocks integrated                              */
   uint64_t seq_rejects;     /* pushes rejected with CORR_ESEQ                 */
   uint64_t dumps;           /* corr_dump calls                                */
-  uint64_t turn_launches;   /* corner-turn kernels launched                   */
+  uint64_t turn_launches;   /* corner-turn (and row-padding) kernels launched */
   uint64_t herk_launches;   /* cross-multiply kernels launched                */
   uint64_t norm_launches;   /* normalisation kernels launched                 */
   double turn_ms;           /* device time in corner-turn kernels (timed)     */

@@ -156,6 +156,12 @@ cudaError_t pkt_turn_launch(const uint8_t* in, uint8_t* out, int n_fids, int inp
 cudaError_t split_planes_launch(const uint8_t* in, uint8_t* out, long long rows, int T,
                                 long long out_stride, cudaStream_t s);
 
+// Rows of T bytes, one after the other at any alignment, copied to rows
+// out_stride bytes apart (a multiple of 32, out 32-byte aligned; the bytes
+// past T of a row's last 32 are undefined).
+cudaError_t pad_rows_launch(const uint8_t* in, uint8_t* out, long long rows, int T,
+                            long long out_stride, cudaStream_t s);
+
 // Lay one block out as [channel][byte row][time] with rows of out_stride
 // bytes (byte rows: one per input at 4 bits, re and im bytes at 8 bits).
 // Returns false without launching when the layout is already that one

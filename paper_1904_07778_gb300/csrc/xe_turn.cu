@@ -409,6 +409,26 @@ __global__ void split_planes_kernel(const uint8_t* __restrict__ in, uint8_t* __r
   }
 }
 
+// ---------------------------------------------------------------- row padding
+// 4-bit [c][i][t] rows of T bytes (any alignment) copied to rows os bytes
+// apart (aligned to and padded to 32 bytes), one 32-byte piece a thread.
+__global__ void pad_rows_kernel(const uint8_t* __restrict__ in, uint8_t* __restrict__ out,
+                                long long rows, int T, long long os) {
+  const int per_row = (T + 31) / 32;
+  const long long total = rows * per_row;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
+       e += (long long)gridDim.x * blockDim.x) {
+    const long long r = e / per_row;
+    const int t = (int)(e - r * per_row) * 32;
+    const uint8_t* src = in + r * T + t;
+    uint32_t a[4], b[4];
+    ld16_any(src, in, in + rows * T, a);
+    ld16_any(src + 16, in, in + rows * T, b);
+    const uint32_t w[8] = {a[0], a[1], a[2], a[3], b[0], b[1], b[2], b[3]};
+    st32B(out + r * os + t, w);
+  }
+}
+
 // ---------------------------------------------------------------- normalise
 // rho = V / sqrt(V_ii V_jj) for a range of one channel's baselines.
 //
@@ -541,6 +561,16 @@ cudaError_t split_planes_launch(const uint8_t* in, uint8_t* out, long long rows,
   if (blocks > 152 * 16) blocks = 152 * 16;
   if (blocks < 1) blocks = 1;
   split_planes_kernel<<<(unsigned)blocks, 256, 0, s>>>(in, out, rows, T, out_stride, vec);
+  return cudaGetLastError();
+}
+
+cudaError_t pad_rows_launch(const uint8_t* in, uint8_t* out, long long rows, int T,
+                            long long out_stride, cudaStream_t s) {
+  if (out_stride % 32 != 0 || out_stride < T || reinterpret_cast<uintptr_t>(out) % 32 != 0)
+    return cudaErrorInvalidValue;
+  const long long blocks = (rows * ((T + 31) / 32) + 255) / 256;
+  pad_rows_kernel<<<(unsigned)std::min<long long>(blocks, device_sm_count() * 64), 256, 0, s>>>(
+      in, out, rows, T, out_stride);
   return cudaGetLastError();
 }
 
