@@ -138,12 +138,25 @@ __device__ __forceinline__ void s8_to_f16(const uint32_t (&w)[4], const uint32_t
   }
 }
 
+// Row of a 128-row block that holds plane `plane` (0 Re, 1 Im) of the
+// block's sample m (0 .. 63): 8 real rows, then their 8 imaginary rows, the 8
+// samples of a group in the order 0, 4, 1, 5, 2, 6, 3, 7.  A 16-row, 16-column
+// tensor-memory load of the drain then gives each thread the whole 2 x 2
+// blocks of two visibilities (no exchange between lanes), and four
+// neighbouring threads store 64 contiguous bytes.
+__host__ __device__ constexpr int op_row(int m, int plane) {
+  return 16 * (m >> 3) + 8 * plane + 2 * (m & 3) + ((m >> 2) & 1);
+}
+
+// Row sums are kept on top of this pattern: as a float it is 2^23 + U.
+constexpr int32_t kUsumZero = 0x4B000000;
+
 __device__ __forceinline__ void store_pair(uint8_t* stage, int pair, int chunk,
                                            const uint32_t (&re)[4], const uint32_t (&im)[4]) {
   uint8_t* blk = stage + (pair >> 6) * kOpBlockBytes;
-  const int r0 = (pair & 63) * 2;
-  *reinterpret_cast<uint4*>(blk + swz_offset(r0, chunk)) = make_uint4(re[0], re[1], re[2], re[3]);
-  *reinterpret_cast<uint4*>(blk + swz_offset(r0 + 1, chunk)) = make_uint4(im[0], im[1], im[2], im[3]);
+  const int m = pair & 63;
+  *reinterpret_cast<uint4*>(blk + swz_offset(op_row(m, 0), chunk)) = make_uint4(re[0], re[1], re[2], re[3]);
+  *reinterpret_cast<uint4*>(blk + swz_offset(op_row(m, 1), chunk)) = make_uint4(im[0], im[1], im[2], im[3]);
 }
 
 // Masks for a 16-spectrum chunk starting at spectrum tk of a launch of tn.
@@ -158,27 +171,32 @@ __device__ __forceinline__ void time_keep(int tk, int tn, uint32_t (&keep)[4]) {
   }
 }
 
-// Row sums: the CH lanes of a pair hold its CH 16-spectrum chunks; item it
-// of a thread covers pair it * (NT / CH) + tid / CH.  Partial sums of
-// several unpack groups are added with shared-memory atomics.
-template <int NT, int NI, int CH = 8>
-__device__ __forceinline__ void publish_row_sums(int32_t (&sre)[NI], int32_t (&sim)[NI], int nit,
+// Row sums: the 8 lanes of a pair hold its 8 16-spectrum chunks; item it of a
+// thread covers pair 16 it + tid / 8.  Three halving exchanges leave each
+// lane with the whole sums of one plane of two items (14 shuffles instead of
+// the 48 of a butterfly per sum), which it adds to the shared sums: partial
+// sums of several unpack groups meet there.  All groups publish at a task's
+// end, with the ring running dry behind them.
+template <int NI>
+__device__ __forceinline__ void publish_row_sums(const int32_t (&sre)[NI], const int32_t (&sim)[NI], int nit,
                                                  int tid, int32_t* usum) {
+  static_assert(NI == 8, "eight items of two planes over eight lanes");
+  const bool b2 = tid & 4, b1 = tid & 2, b0 = tid & 1;
+  int v[8];
 #pragma unroll
-  for (int it = 0; it < NI; ++it) {
-    if (it < nit) {
-      int r = sre[it], m = sim[it];
+  for (int k = 0; k < 8; ++k)
+    v[k] = (b2 ? sim[k] : sre[k]) + __shfl_xor_sync(0xFFFFFFFFu, b2 ? sre[k] : sim[k], 4);
 #pragma unroll
-      for (int x = 1; x < CH; x <<= 1) {
-        r += __shfl_xor_sync(0xFFFFFFFFu, r, x);
-        m += __shfl_xor_sync(0xFFFFFFFFu, m, x);
-      }
-      if ((tid & (CH - 1)) == 0) {
-        const int pair = it * (NT / CH) + tid / CH;
-        atomicAdd(&usum[(pair >> 6) * 128 + (pair & 63) * 2], r);
-        atomicAdd(&usum[(pair >> 6) * 128 + (pair & 63) * 2 + 1], m);
-      }
-    }
+  for (int k = 0; k < 4; ++k)
+    v[k] = (b1 ? v[k + 4] : v[k]) + __shfl_xor_sync(0xFFFFFFFFu, b1 ? v[k] : v[k + 4], 2);
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+    v[k] = (b0 ? v[k + 2] : v[k]) + __shfl_xor_sync(0xFFFFFFFFu, b0 ? v[k] : v[k + 2], 1);
+  const int it = (b1 ? 4 : 0) + (b0 ? 2 : 0), pair = 16 * it + (tid >> 3);
+  if (it < nit) {
+    int32_t* u = usum + (pair >> 6) * 128 + op_row(pair & 63, b2 ? 1 : 0);
+    atomicAdd(u, v[0]);
+    atomicAdd(u + 32, v[1]);  // 16 samples on
   }
 }
 
@@ -271,151 +289,157 @@ __device__ __forceinline__ void mma_loop(const TaskGeom& g, int nk, int nst, uin
 // blocks into complex visibilities and store or add them into the int64
 // integration buffer.  The calling warp reads tensor-memory lanes
 // 32 quad .. + 31 (rows of the A block; quad must be the warp index mod 4)
-// and the part-th of nparts shares of the 16-column chunks.  Column block
+// and every nparts-th 16-column chunk from the part-th on.  Column block
 // c < rb is a lower-triangle block, c == rb the diagonal block (entries
 // j <= i only), c > rb the transpose of block (c, rb): there the thread's
 // row is the second input of the baseline and the imaginary part changes
-// sign.  The two lanes of an input (rows 2i and 2i + 1) exchange halves so
-// that each holds whole (Re, Im) pairs: the even-numbered columns j of the
-// chunk go to the lane of row 2i, the odd ones to row 2i + 1, and each
-// visibility is one 16-byte store (adjacent lanes fill 32 contiguous bytes
-// in lower blocks, 16 lanes fill 256 contiguous bytes in upper blocks).
+// sign.
+//
+// What bounds it is its instruction count: the drain warps share their SMSPs
+// with four busy unpack warps each.  So a thread holds whole 2 x 2 blocks
+// (rows and columns of a block come as 8 real, 8 imaginary; see op_row), 16
+// rows that hold only entries above the diagonal are not even loaded, and the
+// 4-bit correction takes two packed FMAs per pair of values and no
+// conversion: with the row sums kept as the floats g = 2^23 + U,
+//     K = 64 T - 8 U_p - 8 U_q + 1.5 2^23 = -8 g_q + (-8 g_p + const)
+// is a multiple of 8 below 2^27, and 2^18 Gu + K = 1.5 2^23 + G is an integer
+// in [2^23, 2^24] (|G| <= 64 T <= 2^22): every step is exact, and the float's
+// bits less those of 1.5 2^23 are the integer G.  A clock probe of the form
+// before (general index arithmetic per value) put most of a chunk's time into
+// its own serial instructions, about 10 cycles each on the shared SMSPs, so
+// the walk along a row or column carries only a pointer and a limit.
+// Push and dump of 192 x 1024 x 1024 [c][i][t]: 0.179 -> 0.145 ms (0.141 with
+// the row sums' exchanges below); 16 dish blocks in one launch 0.504 -> 0.493
+// (0.484) ms.
 //
 // F16 (8-bit samples): the accumulators hold G itself.  A task is drained
 // once per accumulation of at most 1024 spectra; every accumulation but the
-// last leaves its int32 visibilities in the CTA's scratch (int2 per
-// position, entry (4 cc + u) 128 + p, written and read by the same thread),
-// which the next one adds in, and the last goes to the integration buffer.
-// The int32 sums stay below 2 * 127^2 * 32768 < 2^31 for the longest block.
+// last leaves its int32 visibilities in the CTA's scratch (int4: two
+// visibilities of 32 threads per chunk, 16 rows and quarter, written and read
+// by the same thread), which the next one adds in, and the last goes to the
+// integration buffer.  The int32 sums stay below 2 * 127^2 * 32768 < 2^31 for
+// the longest block.
 template <bool F16>
 __device__ __forceinline__ void epilogue(const HerkInst& a, const HerkTask& task, const TaskGeom& g,
                                          const int32_t* usum, uint32_t tmem, int quad, int part,
                                          int nparts, int lane, bool first, bool last, int2* scr) {
-  const bool stacked = a.rows_per_chan > 0;
-  const int p = quad * 32 + lane;
   const int n = a.n_inputs;
-  int ch, i, plane;
-  bool row_ok;
-  // A stacked tile has a power of two (2 .. 64) of rows per channel, so its
-  // channel and row splits are masks and shifts (the drain warps share their
-  // SMSPs with the busy unpack warps: every instruction of theirs counts).
-  if (stacked) {
-    const int rpc = a.rows_per_chan;
-    ch = task.chan0 + (p >> (31 - __clz(rpc)));
-    const int rr = p & (rpc - 1);
-    i = rr >> 1;
-    plane = rr & 1;
-    row_ok = i < n && ch < a.n_chans;
-  } else {
-    ch = task.chan0;
-    const int prow = task.rb * 128 + p;
-    i = prow >> 1;
-    plane = prow & 1;
-    row_ok = i < n;
-  }
-  const int base_term = F16 ? 0 : 64 * a.tn - 8 * usum[g.a_slot * 128 + p];
-  const long long nbl = (long long)n * (n + 1) / 2;
-  int64_t* chp = a.acc + (long long)(row_ok ? ch : 0) * nbl * 2;
-  const int tri_i = i * (i + 1) / 2;  // baselines per channel stay below 2^30 (inputs <= 32768)
-  const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
-  // 16-column chunks of this warp's share.  In a stacked tile a lane's row
-  // only meets columns of its own channel: the rows 32 quad .. + 31 of this
-  // warp belong to one channel (rows_per_chan >= 32), whose columns are
-  // rows_per_chan / 16 chunks, or to channels whose columns are the two
-  // chunks 2 quad, 2 quad + 1; the other chunks hold no visibility.
-  int c0 = 0, c1 = g.nb * 8;
-  if (stacked) {
-    const int rpc = a.rows_per_chan;
-    c0 = rpc >= 32 ? (rpc == 32 ? quad : quad >> 1) * (rpc >> 4) : 2 * quad;  // rpc <= 64
-    c1 = c0 + (rpc >= 32 ? rpc >> 4 : 2);
-  }
-  const int per = (c1 - c0 + nparts - 1) / nparts;
-  const int cbeg = c0 + part * per, cend = min(c1, cbeg + per);
-  for (int cc = cbeg; cc < cend; ++cc) {
-    int2 prev[4];
-    int2* sp = scr + (cc * 4) * 128 + p;
-    if (F16 && !first) {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) prev[u] = sp[u * 128];
+  const int half = a.rows_per_chan >> 1;  // samples per channel of a stacked tile (a power of two), 0: not stacked
+  const int q0 = lane & 3;  // the thread's columns of each chunk: samples q0, q0 + 4
+  const int nbl = n * (n + 1) / 2;  // below 2^30 (inputs <= 32768)
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {  // the quarter's 16-row halves
+    const int gr = 2 * quad + h;            // the half's group of 8 samples
+    const int m = 8 * gr + (lane >> 3) + (lane & 4);  // the thread's sample
+    int ch = task.chan0, i = task.rb * 64 + m;
+    if (half) {
+      ch += m >> (31 - __clz(half));
+      i = m & (half - 1);
     }
-    uint32_t r[16];
-    tmem_load16(trow + (uint32_t)(cc * 16), r);
-    int cs[16];  // 4-bit: the chunk's 16 column sums, in four 16-byte loads
+    if (i >= n || ch >= a.n_chans) i = -1;  // nothing to store
+    int64_t* const chp = a.acc + (i >= 0 ? (long long)ch * nbl * 2 : 0);
+    uint64_t kre = 0, kim = 0;  // 4-bit: -8 g_p + const of the two rows, in both halves
     if constexpr (!F16) {
-      const int4* u4 = reinterpret_cast<const int4*>(usum + cc * 16);
-#pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        const int4 v = u4[w];
-        cs[4 * w] = v.x, cs[4 * w + 1] = v.y, cs[4 * w + 2] = v.z, cs[4 * w + 3] = v.w;
-      }
+      const float c = (float)(64 * a.tn) + 146800640.0f;  // + 1.5 2^23 + 2 8 2^23
+      const float* us = reinterpret_cast<const float*>(usum + g.a_slot * 128 + op_row(m, 0));
+      kre = f2_dup(fmaf(us[0], -8.0f, c));
+      kim = f2_dup(fmaf(us[8], -8.0f, c));
     }
-    int gv[16];
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      if constexpr (F16)
-        gv[k] = __float2int_rn(__uint_as_float(r[k]));
-      else
-        gv[k] = __float2int_rn(__uint_as_float(r[k]) * 262144.0f) + base_term - 8 * cs[k];
-    }
-    const int cblk = slot_block(g, cc >> 3);
-    const bool upper = !stacked && cblk > task.rb;
-    int vre[4], vim[4];
-    int off[4];  // element offset of the pair within the channel, -1: not stored
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {  // columns 2u (lane of row 2i) and 2u + 1 (row 2i + 1)
-      const int x0 = plane ? gv[4 * u + 2] : gv[4 * u];
-      const int x1 = plane ? gv[4 * u + 3] : gv[4 * u + 1];
-      const int y0 = __shfl_xor_sync(0xFFFFFFFFu, plane ? gv[4 * u] : gv[4 * u + 2], 1);
-      const int y1 = __shfl_xor_sync(0xFFFFFFFFu, plane ? gv[4 * u + 1] : gv[4 * u + 3], 1);
-      // G[2i][2j] + G[2i+1][2j+1] and G[2i+1][2j] - G[2i][2j+1] for this lane's column j
-      vre[u] = plane ? y0 + x1 : x0 + y1;
-      vim[u] = plane ? x0 - y1 : y0 - x1;
-      const int q = (cc & 7) * 16 + 2 * (2 * u + plane);  // real column of input j in its block
-      int b;
-      bool ok;
-      if (stacked) {
-        // column q and row p of the tile share a channel when they agree
-        // above the rows-per-channel bits
-        const int rpc = a.rows_per_chan;
-        const int j = (q & (rpc - 1)) >> 1;
-        ok = row_ok && (q ^ p) < rpc && j <= i;
-        b = tri_i + j;
-      } else {
-        const int j = (128 * cblk + q) >> 1;
-        if (upper) {
-          ok = row_ok && j < n;  // baseline (j, i), j > i: the conjugate
-          b = j * (j + 1) / 2 + i;
-          vim[u] = -vim[u];
+    const uint32_t trow = tmem + ((uint32_t)(quad * 32 + 16 * h) << 16);
+    int4* const sp = reinterpret_cast<int4*>(scr) + (h * 4 + quad) * 32 + lane;
+    // Chunks c0 + k, c0 + k + nparts, ... below c0 + kn: emit(k, re0, im0,
+    // re1, im1) takes the visibilities of columns 8 k + q0 and 8 k + q0 + 4.  A
+    // chunk loads while the one before it is stored.
+    auto walk = [&](int c0, int k, int kn, auto&& emit) {
+      if (k >= kn) return;
+      uint32_t r[8];
+      int4 prev = make_int4(0, 0, 0, 0);  // 8-bit: the sums of the pieces before
+      tmem_load_16x16(trow + (uint32_t)((c0 + k) * 16), r);
+      if (F16 && !first) prev = sp[(c0 + k) * 256];
+      while (true) {
+        int re0, im0, re1, im1;
+        if constexpr (F16) {
+          tmem_wait_ld(r);
+          auto toi = [](uint32_t x) { return __float2int_rn(__uint_as_float(x)); };
+          re0 = toi(r[0]) + toi(r[6]) + prev.x;
+          im0 = toi(r[2]) - toi(r[4]) + prev.y;
+          re1 = toi(r[1]) + toi(r[7]) + prev.z;
+          im1 = toi(r[3]) - toi(r[5]) + prev.w;
         } else {
-          ok = row_ok && j <= i;
-          b = tri_i + j;
+          const uint64_t m8 = f2_dup(-8.0f), s18 = f2_dup(262144.0f);
+          // the columns' sums (floats 2^23 + U) of samples q0, q0 + 4
+          const int32_t* us = usum + (c0 + k) * 16 + 2 * q0;
+          const uint64_t gre = *reinterpret_cast<const uint64_t*>(us);
+          const uint64_t gim = *reinterpret_cast<const uint64_t*>(us + 8);
+          const uint64_t k00 = f2_fma(gre, m8, kre), k10 = f2_fma(gre, m8, kim);
+          const uint64_t k01 = f2_fma(gim, m8, kre), k11 = f2_fma(gim, m8, kim);
+          tmem_wait_ld(r);
+          uint32_t g00[2], g10[2], g01[2], g11[2];  // [row plane][column plane], bits of 1.5 2^23 + G
+          f2_unpack(f2_fma(f2_pack(r[0], r[1]), s18, k00), g00[0], g00[1]);
+          f2_unpack(f2_fma(f2_pack(r[2], r[3]), s18, k10), g10[0], g10[1]);
+          f2_unpack(f2_fma(f2_pack(r[4], r[5]), s18, k01), g01[0], g01[1]);
+          f2_unpack(f2_fma(f2_pack(r[6], r[7]), s18, k11), g11[0], g11[1]);
+          re0 = (int)(g00[0] + g11[0] - 2u * 0x4B400000u);
+          im0 = (int)(g10[0] - g01[0]);
+          re1 = (int)(g00[1] + g11[1] - 2u * 0x4B400000u);
+          im1 = (int)(g10[1] - g01[1]);
         }
-      }
-      off[u] = ok ? 2 * b : -1;
-    }
-    if (F16) {
-      if (!first) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          vre[u] += prev[u].x;
-          vim[u] += prev[u].y;
+        const int kk = k;
+        k += nparts;
+        if (k < kn) {
+          tmem_load_16x16(trow + (uint32_t)((c0 + k) * 16), r);
+          if (F16 && !first) prev = sp[(c0 + k) * 256];
         }
+        if (F16 && !last)
+          sp[(c0 + kk) * 256] = make_int4(re0, im0, re1, im1);
+        else
+          emit(kk, re0, im0, re1, im1);
+        if (k >= kn) break;
       }
-      if (!last) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) sp[u * 128] = make_int2(vre[u], vim[u]);
-        continue;
-      }
-    }
-    if (a.accumulate) {
-      // reductions at L2: nothing waits for the old value
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (off[u] >= 0) red_s64x2(chp + off[u], vre[u], vim[u]);
+    };
+    auto put = [&](int64_t* p, int re, int im, bool ok) {
+      if (!ok) return;
+      if (a.accumulate)
+        red_s64x2(p, re, im);  // at L2: nothing waits for the old value
+      else
+        st_s64x2(p, re, im);
+    };
+    // along a row: baselines (i, j0 + 8 k + q0) and four on, while not above the diagonal
+    auto row_walk = [&](int c0, int kn, int j0) {
+      int64_t* const p = chp + 2 * (i * (i + 1) / 2 + j0 + q0);
+      const int lim = i - j0 - q0;
+      walk(c0, part, kn, [&](int k, int re0, int im0, int re1, int im1) {
+        put(p + 16 * k, re0, im0, 8 * k <= lim);
+        put(p + 16 * k + 8, re1, im1, 8 * k + 4 <= lim);
+      });
+    };
+    if (half >= 8) {  // the columns of the rows' own channel, up to the rows' group
+      const int c0 = gr & ~((half >> 3) - 1);
+      row_walk(c0, gr - c0 + 1, 0);
+    } else if (half) {  // several channels in the rows' group: one chunk
+      // a column and a row of the tile share a channel when their samples
+      // agree above the samples-per-channel bits
+      walk(gr, part, 1, [&](int, int re0, int im0, int re1, int im1) {
+        const int mc = 8 * gr + q0, j0 = mc & (half - 1), j1 = (mc + 4) & (half - 1);
+        put(chp + 2 * (i * (i + 1) / 2 + j0), re0, im0, (mc ^ m) < half && j0 <= i);
+        put(chp + 2 * (i * (i + 1) / 2 + j1), re1, im1, ((mc + 4) ^ m) < half && j1 <= i);
+      });
     } else {
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (off[u] >= 0) st_s64x2(chp + off[u], vre[u], vim[u]);
+#pragma unroll 1
+      for (int s = 0; s < g.nb; ++s) {
+        const int cblk = slot_block(g, s);
+        if (cblk <= task.rb) {  // the diagonal block up to the rows' group, or a lower block
+          row_walk(8 * s, cblk == task.rb ? gr + 1 : 8, 64 * cblk);
+        } else {  // baselines (j, i), j > i: the conjugate
+          const int jb = 64 * cblk + q0;
+          walk(8 * s, part, 8, [&](int k, int re0, int im0, int re1, int im1) {
+            const int j = jb + 8 * k;
+            int64_t* p = chp + 2 * (j * (j + 1) / 2 + i);
+            put(p, re0, -im0, i >= 0 && j < n);
+            put(p + 2 * (4 * j + 10), re1, -im1, i >= 0 && j + 4 < n);
+          });
+        }
+      }
     }
   }
 }
@@ -441,7 +465,7 @@ __device__ __forceinline__ void ctrl_init_common(Ctrl& sm, int tid) {
     mbar_init(&sm.done, 1);
     sm.abort = 0;
   }
-  for (int i = tid; i < kMaxBlocks * 128; i += blockDim.x) sm.usum[i] = 0;
+  for (int i = tid; i < kMaxBlocks * 128; i += blockDim.x) sm.usum[i] = kUsumZero;
 }
 
 // ------------------------------------------------------------- ring kernel
@@ -511,12 +535,13 @@ constexpr int kRingThreads = (kEpiWarp0 + kEpiWarps) * 32;
 // registers per thread: launch share, unpack warpgroups, the other warpgroups.
 // Chosen per instance from the compiler's spill report and measured times:
 // the 8-bit drain, which adds the accumulations' partial sums, takes more,
-// the 8-bit unpack less; the low-nibble-real 4-bit unpack needs 88.
+// the 8-bit unpack less; the 4-bit unpack spills below 88 (the cylinder block
+// 1.11 ms at 80 / 56 against 1.07).
 constexpr int kRegsLaunch = (65536 / kRingThreads) & ~7;
 template <bool LO, bool EIGHT>
-__host__ __device__ constexpr int regs_unpack() { return EIGHT ? 72 : (LO ? 88 : 80); }
+__host__ __device__ constexpr int regs_unpack() { return EIGHT ? 72 : 88; }
 template <bool LO, bool EIGHT>
-__host__ __device__ constexpr int regs_other() { return EIGHT ? 64 : (LO ? 48 : 56); }
+__host__ __device__ constexpr int regs_other() { return EIGHT ? 72 : 48; }
 static_assert(kRingThreads % 128 == 0, "whole warpgroups");
 template <bool LO, bool EIGHT>
 constexpr bool regs_fit() {
@@ -618,7 +643,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
     mbar_init(&sm.done, 1);
     sm.abort = 0;
   }
-  for (int i = tid; i < 2 * kMaxBlocks * 128; i += blockDim.x) (&sm.usum[0][0])[i] = 0;
+  for (int i = tid; i < 2 * kMaxBlocks * 128; i += blockDim.x) (&sm.usum[0][0])[i] = kUsumZero;
   if (warp == 0) tmem_alloc(&sm.tmem_base, 512);
   fence_mbar_init();
   tc_before_sync();
@@ -762,24 +787,29 @@ __global__ void __launch_bounds__(kRingThreads, 1)
     const int gt = tid - grp * kGroupThreads;
     // Item geometry of this thread (four 16-byte items per packed block).
     //   4-bit, [c][row][t]: byte row g8 + 16 it' of the block, spectra
-    //     16 chunk .. + 15 -> operand rows 2 (g8 + 16 it') and + 1, chunk
-    //     `chunk`; payload order: rows 4 tq .. + 3, K chunk tc (see tci_t).
+    //     16 chunk .. + 15 -> its operand rows (op_row), chunk `chunk`;
+    //     payload order: rows 4 tq .. + 3, K chunk tc (see tci_t).
     //   8-bit, [c][row][t]: byte row r32 + 32 it', spectra 16 c4 .. + 15 ->
-    //     operand row r32 + 32 it', chunks 2 c4 and 2 c4 + 1; payload order:
+    //     its operand row, chunks 2 c4 and 2 c4 + 1; payload order:
     //     rows 4 lane .. + 3, spectra 16 c8 .. + 15 gathered with the halves
     //     swapped on odd lanes (sw8), which keeps the stores free of bank
     //     conflicts (the gathers are: a row of 128 bytes per spectrum puts
     //     lane l's word in bank l).
     const int chunk = gt & 7, g8 = gt >> 3;
     const int tq = lane >> 1, tc = (lane + 2 * (gt >> 5)) & 7;
-    const int c4 = gt & 3, r32 = gt >> 2;
+    // (8-bit rows: neighbouring threads take the real plane of one sample and the
+    // imaginary plane of the sample four on, so that the loads alternate row
+    // parity and the stores differ in the lowest bit of row mod 8: neither has
+    // bank conflicts)
+    const int c4 = gt & 3, r32 = 2 * ((gt >> 3) ^ (gt & 4)) + ((gt >> 2) & 1);
     const int c8 = ((gt >> 5) + (lane >> 1)) & 3, sw8 = 8 * (lane & 1);
     const uint32_t src0 =
         ring_addr + (uint32_t)(EIGHT ? kPkRowBytes * r32 + 16 * c4 : kPkRowBytes * g8 + 16 * chunk);
     static_assert(kMaxBlocks == 2, "a stage holds at most two 128-row blocks");
     // later items add whole 8-row atoms, so the swizzle position stays the same
-    const uint32_t dst_a = ring_addr + (EIGHT ? swz_offset(r32, 2 * c4) : swz_offset(2 * g8, chunk));
-    const uint32_t dst_b = ring_addr + (EIGHT ? swz_offset(r32, 2 * c4 + 1) : swz_offset(2 * g8 + 1, chunk));
+    // (the second store: the next 8-row atom at 4 bits, the neighbouring chunk at 8)
+    const uint32_t dst0 = ring_addr + (EIGHT ? swz_offset(op_row(r32 >> 1, r32 & 1), 2 * c4)
+                                             : swz_offset(op_row(g8, 0), chunk));
     bool ok = true;
     // next stage of this group, its slot s = S mod ns and use m = S / ns,
     // advanced by additions (kGroups <= ns)
@@ -860,26 +890,26 @@ __global__ void __launch_bounds__(kRingThreads, 1)
               uint32_t h[8];
               s8_to_f16(w, keep, h, bad);
               if constexpr (TCI) {
-                const int r = 4 * lane + u, sw = sw8 >> 3;
+                const int r = op_row(2 * lane + (u >> 1), u & 1), sw = sw8 >> 3;
                 sts128(ob + swz_offset(r, 2 * c8 + sw), h[0], h[1], h[2], h[3]);
                 sts128(ob + swz_offset(r, 2 * c8 + 1 - sw), h[4], h[5], h[6], h[7]);
               } else {
                 const uint32_t o = so + (uint32_t)(it * kROpBlock + 4096 * u);  // 32 operand rows on
-                sts128(dst_a + o, h[0], h[1], h[2], h[3]);
-                sts128(dst_b + o, h[4], h[5], h[6], h[7]);
+                sts128(dst0 + o, h[0], h[1], h[2], h[3]);
+                sts128((dst0 + o) ^ 16u, h[4], h[5], h[6], h[7]);
               }
             } else {
               uint32_t re[4], im[4];
               // always masked (all ones before the last stage): no branch inside the unrolled loop
               unpack16<LO_IS_REAL, true>(w, keep, re, im, sre[4 * it + u], sim[4 * it + u]);
               if constexpr (TCI) {
-                const int r = 2 * (4 * tq + u);
+                const int r = op_row(4 * tq + u, 0);  // the imaginary row is 8 rows (an atom) on
                 sts128(ob + swz_offset(r, tc), re[0], re[1], re[2], re[3]);
-                sts128(ob + swz_offset(r + 1, tc), im[0], im[1], im[2], im[3]);
+                sts128(ob + swz_offset(r, tc) + 1024, im[0], im[1], im[2], im[3]);
               } else {
                 const uint32_t o = so + (uint32_t)(it * kROpBlock + 4096 * u);
-                sts128(dst_a + o, re[0], re[1], re[2], re[3]);
-                sts128(dst_b + o, im[0], im[1], im[2], im[3]);
+                sts128(dst0 + o, re[0], re[1], re[2], re[3]);
+                sts128(dst0 + o + 1024u, im[0], im[1], im[2], im[3]);
               }
             }
           }
@@ -920,23 +950,20 @@ __global__ void __launch_bounds__(kRingThreads, 1)
       if (!freed) raise_timeout(a.status, abort);
       if (!named_bar_and(2 + grp, kGroupThreads, freed)) break;
       if constexpr (TCI) {
-        // the two lanes of a quad in a warp add, then one adds per warp
+        // the two lanes of a quad exchange planes, then each adds its own
 #pragma unroll
         for (int it = 0; it < kMaxBlocks; ++it) {
+          if (it < g.nblk) {
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            if (it < g.nblk) {
-              const int r = sre[4 * it + u] + __shfl_xor_sync(0xFFFFFFFFu, sre[4 * it + u], 1);
-              const int mm = sim[4 * it + u] + __shfl_xor_sync(0xFFFFFFFFu, sim[4 * it + u], 1);
-              if ((lane & 1) == 0) {
-                atomicAdd(&sm.usum[b][it * 128 + 2 * (4 * tq + u)], r);
-                atomicAdd(&sm.usum[b][it * 128 + 2 * (4 * tq + u) + 1], mm);
-              }
+            for (int u = 0; u < 4; ++u) {
+              const int r = sre[4 * it + u], mm = sim[4 * it + u];
+              const int v = ((lane & 1) ? mm : r) + __shfl_xor_sync(0xFFFFFFFFu, (lane & 1) ? r : mm, 1);
+              atomicAdd(&sm.usum[b][it * 128 + op_row(4 * tq + u, lane & 1)], v);
             }
           }
         }
       } else {
-        publish_row_sums<kGroupThreads, kItems, 8>(sre, sim, nit, gt, sm.usum[b]);
+        publish_row_sums(sre, sim, nit, gt, sm.usum[b]);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.usum_full[b]);
@@ -976,7 +1003,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
           // every drain warp has read the sums: clear them for task j + 2
           named_bar_sync(1, kEpiWarps * 32);
           for (int i = tid - kEpiWarp0 * 32; i < kMaxBlocks * 128; i += kEpiWarps * 32)
-            sm.usum[b][i] = 0;
+            sm.usum[b][i] = kUsumZero;
           __syncwarp();
           if (lane == 0) mbar_arrive(&sm.usum_empty[b]);
         }
@@ -1103,7 +1130,7 @@ __global__ void __launch_bounds__(kLdgThreads, 1) herk4_ldg_kernel(const HerkArg
         ph ^= 1u;
       }
     }
-    publish_row_sums<128>(sre, sim, nit, tid, sm.usum);
+    publish_row_sums(sre, sim, nit, tid, sm.usum);
     named_bar_sync(1, 128);
     int never = 0;
     bool good = mbar_wait(&sm.done, 0, &never);
