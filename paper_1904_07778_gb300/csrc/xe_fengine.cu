@@ -3,14 +3,14 @@
 // output, and the equaliser / requantiser to packed fix_4_3 codes -- one
 // fused kernel whose output is the X-engine's input.
 //
-// A CTA takes one input pair (2k, 2k+1) and a group of 32 consecutive
-// spectra.  Per spectrum, M/8 threads (an "FFT unit"; a CTA holds
-// 2048/M units for M <= 2048) filter 8 consecutive samples each, store
-// z[n] = y_2k[n] + j y_2k+1[n] in padded shared memory, and run an in-place
-// Stockham FFT (radix-8 passes, then one radix-2 or radix-4 pass).  The
-// separated spectra are rounded to 18 bits, equalised, packed, and staged
-// as [channel][input][spectrum] so that the group leaves as 32-byte runs of
-// the X-engine's [c][i][t] order: the corner turn happens here.
+// A CTA takes one input pair (2k, 2k+1) and a group of consecutive spectra.
+// M/8 threads (an "FFT unit"; a CTA holds 2048/M units for M <= 2048, each
+// with its own stretch of the group) take two spectra at a time: they filter 8 consecutive samples
+// each, store z[n] = y_2k[n] + j y_2k+1[n] of both in padded shared memory,
+// and run in-place Stockham FFTs (radix-8 passes, then one radix-2 or radix-4
+// pass).  The separated spectra are rounded to 18 bits, equalised, packed, and
+// staged per thread until 16 spectra of its channels leave as 16-byte pieces
+// of the X-engine's [c][i][t] order: the corner turn happens here.
 #include <algorithm>
 #include <cmath>
 #include <new>
@@ -33,11 +33,6 @@ struct fe_ctx {
 namespace xe {
 namespace {
 
-constexpr int kFeGroup = 32;  // spectra per CTA
-// spectra a unit transforms side by side (they share the pass barriers);
-// three measured no faster than two
-__host__ __device__ constexpr int fe_nb(int) { return 2; }
-
 struct FeArgs {
   const int8_t* adc;
   long long adc_stride;
@@ -50,6 +45,7 @@ struct FeArgs {
   float* spec;
   unsigned long long* power;
   int n_inputs, n_spectra, taps, layout;
+  int per_unit;  // consecutive spectra of each FFT unit: 2, 4, 8, 16 or 32
   int lo_is_real, vec_in, vec_out;
   float scale;  // 2^-(shift + 1): Eq. 2's halving and the 18-bit scaling
 };
@@ -57,57 +53,111 @@ struct FeArgs {
 __host__ __device__ constexpr int fe_threads(int logm) {
   return (1 << logm) / 8 > 256 ? (1 << logm) / 8 : 256;
 }
-// one float2 of padding per 16: consecutive runs of 16 (half a warp's
-// 8-byte accesses) stay contiguous, stride-8 runs spread over the banks
-__host__ __device__ constexpr int fe_pad(int n) { return n + (n >> 4); }
+// One point of padding (16 bytes: both spectra's complex values) per 8 and
+// another per 64: aligned runs of 8 points (a quarter-warp's 16-byte accesses)
+// stay contiguous, and runs of stride 8 and 64 spread over the banks.
+__host__ __device__ constexpr int fe_pad(int n) { return n + (n >> 3) + (n >> 6); }
 // Twiddles of the radix-8 passes at Ns = 8 and Ns = 64 in shared memory,
-// [k][j-1] for k < Ns: they depend only on lt mod Ns, so the table is small
-// (threads with equal k read the same entry) and frees the registers they
-// would take.
+// [k][j-1] for k < Ns, each value twice: they depend only on lt mod Ns, so
+// the table is small (threads with equal k read the same entry) and frees the
+// registers they would take.  Row k of the Ns = 64 part lies at
+// 8 (k mod 8) + k / 8: the threads of a class (below) read neighbouring rows.
 constexpr int kTwTable = (8 + 64) * 7;
+__host__ __device__ constexpr int tw64_row(int k) { return 8 * (k & 7) + (k >> 3); }
+__host__ __device__ constexpr int fe_units(int logm) { return fe_threads(logm) / ((1 << logm) / 8); }
+// Codes staged per thread before they leave: its four channels of up to 16
+// spectra, two spectra of both inputs to a word.  Only the thread itself reads
+// them back.
+constexpr int kStageIts = 8;
 template <int LOGM>
 constexpr size_t fe_smem_bytes() {
   constexpr int M = 1 << LOGM;
-  constexpr int units = fe_threads(LOGM) / (M / 8);
-  return (size_t)fe_nb(LOGM) * units * fe_pad(M) * sizeof(float2) + (size_t)(M / 2) * 2 * kFeGroup +
-         kTwTable * sizeof(float2);
+  return (size_t)fe_units(LOGM) * fe_pad(M) * 16 + kTwTable * 16 +
+         (size_t)fe_threads(LOGM) * 4 * (kStageIts * sizeof(uint32_t) + sizeof(float2) + sizeof(uint32_t));
 }
 
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-  return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+// ---- two spectra side by side -------------------------------------------------
+// A unit transforms two consecutive spectra at once, and every value of the
+// FFT, the separation and the equaliser is a pair of FP32 numbers, one per
+// spectrum, in packed instructions (each half rounded as the scalar
+// operation would be): half the instructions to issue for the same FP32
+// work, and one 16-byte shared-memory access per point of both spectra.
+struct C2 {
+  uint64_t x, y;  // real and imaginary parts of the two spectra
+};
+__device__ __forceinline__ uint64_t p_pack(float a, float b) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+  return d;
 }
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ float2 mul_mj(float2 a) { return make_float2(a.y, -a.x); }  // a * (-j)
+__device__ __forceinline__ void p_unpack(uint64_t v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t p_dup(float a) { return p_pack(a, a); }
+__device__ __forceinline__ uint64_t p_add(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t p_sub(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t p_mul(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t p_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t p_neg(uint64_t a) {
+  float x, y;
+  p_unpack(a, x, y);
+  return p_pack(-x, -y);
+}
+
+// a b with b's parts given twice each
+__device__ __forceinline__ C2 cmul(const C2& a, uint64_t bx, uint64_t by) {
+  return {p_fma(a.x, bx, p_neg(p_mul(a.y, by))), p_fma(a.x, by, p_mul(a.y, bx))};
+}
+__device__ __forceinline__ C2 cadd(const C2& a, const C2& b) { return {p_add(a.x, b.x), p_add(a.y, b.y)}; }
+__device__ __forceinline__ C2 csub(const C2& a, const C2& b) { return {p_sub(a.x, b.x), p_sub(a.y, b.y)}; }
+// a - j b and a + j b
+__device__ __forceinline__ C2 csub_j(const C2& a, const C2& b) { return {p_add(a.x, b.y), p_sub(a.y, b.x)}; }
+__device__ __forceinline__ C2 cadd_j(const C2& a, const C2& b) { return {p_sub(a.x, b.y), p_add(a.y, b.x)}; }
 
 // Y[k] = sum_n x[n] (-j)^(nk)
-__device__ __forceinline__ void dft4(float2& x0, float2& x1, float2& x2, float2& x3) {
-  const float2 t0 = cadd(x0, x2), t1 = csub(x0, x2), t2 = cadd(x1, x3), t3 = mul_mj(csub(x1, x3));
+__device__ __forceinline__ void dft4(C2& x0, C2& x1, C2& x2, C2& x3) {
+  const C2 t0 = cadd(x0, x2), t1 = csub(x0, x2), t2 = cadd(x1, x3), t3 = csub(x1, x3);
   x0 = cadd(t0, t2);
   x2 = csub(t0, t2);
-  x1 = cadd(t1, t3);
-  x3 = csub(t1, t3);
+  x1 = csub_j(t1, t3);
+  x3 = cadd_j(t1, t3);
 }
 
 // X[k] = sum_n a[n] W8^(nk), W8 = exp(-j pi / 4): two DFT4s of the even and
-// odd samples, joined with W8^k.
-__device__ __forceinline__ void dft8(float2 (&a)[8]) {
-  float2 e0 = a[0], e1 = a[2], e2 = a[4], e3 = a[6];
-  float2 o0 = a[1], o1 = a[3], o2 = a[5], o3 = a[7];
+// odd samples, joined with W8^k.  The factors 1/sqrt2 of W8 and W8^3 go into
+// fused multiply-adds with the sums and differences they scale.
+__device__ __forceinline__ void dft8(C2 (&a)[8]) {
+  C2 e0 = a[0], e1 = a[2], e2 = a[4], e3 = a[6];
+  C2 o0 = a[1], o1 = a[3], o2 = a[5], o3 = a[7];
   dft4(e0, e1, e2, e3);
   dft4(o0, o1, o2, o3);
-  const float r = 0.70710678118654752f;
-  o1 = make_float2(r * (o1.x + o1.y), r * (o1.y - o1.x));    // * (1 - j) / sqrt2
-  o2 = mul_mj(o2);                                           // * -j
-  o3 = make_float2(r * (o3.y - o3.x), -r * (o3.x + o3.y));   // * (-1 - j) / sqrt2
+  const uint64_t r = p_dup(0.70710678118654752f), mr = p_dup(-0.70710678118654752f);
   a[0] = cadd(e0, o0);
   a[4] = csub(e0, o0);
-  a[1] = cadd(e1, o1);
-  a[5] = csub(e1, o1);
-  a[2] = cadd(e2, o2);
-  a[6] = csub(e2, o2);
-  a[3] = cadd(e3, o3);
-  a[7] = csub(e3, o3);
+  const uint64_t s1 = p_add(o1.x, o1.y), d1 = p_sub(o1.y, o1.x);  // W8 o1 = r (s1 + j d1)
+  a[1] = {p_fma(r, s1, e1.x), p_fma(r, d1, e1.y)};
+  a[5] = {p_fma(mr, s1, e1.x), p_fma(mr, d1, e1.y)};
+  a[2] = csub_j(e2, o2);
+  a[6] = cadd_j(e2, o2);
+  const uint64_t d3 = p_sub(o3.y, o3.x), s3 = p_add(o3.x, o3.y);  // W8^3 o3 = r (d3 - j s3)
+  a[3] = {p_fma(r, d3, e3.x), p_fma(mr, s3, e3.y)};
+  a[7] = {p_fma(mr, d3, e3.x), p_fma(r, s3, e3.y)};
 }
 
 // Twiddles of one Stockham pass for one thread: butterfly b = lt + r M/8
@@ -115,168 +165,200 @@ __device__ __forceinline__ void dft8(float2 (&a)[8]) {
 // j = 1 .. R-1.  They do not depend on the spectrum, so a thread loads them
 // once (from the FP64-rounded table) and keeps them in registers.
 template <int M, int R>
-__device__ __forceinline__ void load_twiddles(float2 (&tw)[7], int lt, int Ns,
+__device__ __forceinline__ void load_twiddles(float2 (&tw)[7], const int (&b)[8 / R], int Ns,
                                               const float2* __restrict__ w) {
-  constexpr int B = 8 / R;
 #pragma unroll
-  for (int r = 0; r < B; ++r) {
-    const int k = (lt + r * (M / 8)) & (Ns - 1);
-    const int step = k * (M / (R * Ns));
+  for (int r = 0; r < 8 / R; ++r) {
+    const int step = (b[r] & (Ns - 1)) * (M / (R * Ns));
 #pragma unroll
     for (int j = 1; j < R; ++j) tw[r * (R - 1) + j - 1] = __ldg(&w[j * step]);
   }
 }
 
-// One Stockham pass of radix R over NB independent M-point transforms held
-// in zs[] (padded indices): butterfly b reads z[b + j M/R], applies its
-// twiddles, and writes the R outputs to (b div Ns) Ns R + (b mod Ns) + r Ns.
-// Each of the M/8 threads of a unit runs 8/R butterflies per transform;
-// loads and stores are separated by a CTA barrier that the NB transforms
-// share.
-template <int M, int R, int NB, bool STW = false>
-__device__ __forceinline__ void fft_pass(float2* const (&zs)[NB], int lt, int Ns,
-                                         const float2 (&tw)[7], const float2* stw = nullptr) {
+// The butterflies of a thread in a last pass of radix R = 4 or 2 (Ns = M/R,
+// outputs b + r Ns): pairs b and Ns - b, whose outputs are each other's
+// mirror images M - nu, so that the separation of Eq. 2 happens in registers
+// (a pass over shared memory and two barriers less).  b = 0 and b = Ns/2 are
+// their own mirrors: thread 0 takes both.
+template <int M, int R>
+__device__ __forceinline__ void last_butterflies(int lt, int (&b)[8 / R]) {
+  constexpr int Ns = M / R;
+#pragma unroll
+  for (int p = 0; p < 4 / R; ++p) {
+    b[2 * p] = lt + p * (M / 8);
+    b[2 * p + 1] = p == 0 && lt == 0 ? Ns / 2 : Ns - b[2 * p];
+  }
+}
+
+__device__ __forceinline__ C2 z_load(const ulonglong2* z, int i) {
+  const ulonglong2 v = z[i];
+  return {v.x, v.y};
+}
+__device__ __forceinline__ void z_store(ulonglong2* z, int i, const C2& v) {
+  z[i] = make_ulonglong2(v.x, v.y);
+}
+
+// The TPU threads of an FFT unit meet (units are whole warps, or parts of one).
+template <int TPU, int NT>
+__device__ __forceinline__ void unit_sync(int u) {
+  if constexpr (TPU == NT)
+    __syncthreads();
+  else if constexpr (TPU > 32)
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + u), "n"(TPU) : "memory");
+  else
+    __syncwarp();
+}
+
+// The points of a unit with equal index mod 8 form a class: every radix-8 pass
+// after the first maps a class onto itself.  The TPU / 8 threads lt / (TPU/8)
+// = w of the unit take class w's butterflies in those passes and meet among
+// themselves: within a warp (M <= 2048), or 64 threads (M = 4096).
+template <int TPU>
+__device__ __forceinline__ void class_sync(int lt) {
+  if constexpr (TPU / 8 > 32)
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + lt / (TPU / 8)), "n"(TPU / 8) : "memory");
+  else
+    __syncwarp();
+}
+template <int TPU>
+__device__ __forceinline__ int class_butterfly(int lt) {
+  constexpr int n = TPU >= 8 ? TPU / 8 : 1;
+  return 8 * (lt % n) + lt / n;
+}
+
+// Butterflies b[] of a Stockham pass of radix R over a unit's M-point
+// transforms in z (padded indices): butterfly b reads z[b + j M/R], applies
+// its twiddles (registers, or the shared table), and leaves its R outputs in v.
+template <int M, int R, bool STW = false>
+__device__ __forceinline__ void butterflies(C2 (&v)[8], const ulonglong2* z, const int (&bf)[8 / R], int Ns,
+                                            const float2 (&tw)[7], const ulonglong2* stw = nullptr) {
   constexpr int B = 8 / R;       // butterflies per thread
   constexpr int S = M / R;       // input stride
-  float2 v[NB][8];
 #pragma unroll
-  for (int e = 0; e < NB; ++e) {
+  for (int r = 0; r < B; ++r) {
+    const int b = bf[r];
+    const int pb = fe_pad(b);
 #pragma unroll
-    for (int r = 0; r < B; ++r) {
-      const int b = lt + r * (M / 8);
+    for (int j = 0; j < R; ++j)
+      v[r * R + j] = z_load(z, S % 64 == 0 ? pb + j * fe_pad(S) : fe_pad(b + j * S));
+    if (Ns > 1) {
+      const int k = b & (Ns - 1);
+      const ulonglong2* row = STW ? stw + (Ns == 64 ? tw64_row(k) : k) * 7 : nullptr;
 #pragma unroll
-      for (int j = 0; j < R; ++j) v[e][r * R + j] = zs[e][fe_pad(b + j * S)];
-      if (Ns > 1) {
+      for (int j = 1; j < R; ++j) {
         if constexpr (STW) {  // radix 8, one butterfly per thread: this thread's row of the table
-          const float2* row = stw + (b & (Ns - 1)) * 7;
-#pragma unroll
-          for (int j = 1; j < R; ++j) v[e][r * R + j] = cmul(v[e][r * R + j], row[j - 1]);
+          const ulonglong2 t = row[j - 1];
+          v[r * R + j] = cmul(v[r * R + j], t.x, t.y);
         } else {
-#pragma unroll
-          for (int j = 1; j < R; ++j) v[e][r * R + j] = cmul(v[e][r * R + j], tw[r * (R - 1) + j - 1]);
+          const float2 t = tw[r * (R - 1) + j - 1];
+          v[r * R + j] = cmul(v[r * R + j], p_dup(t.x), p_dup(t.y));
         }
       }
     }
-    if constexpr (R == 8) {
-      dft8(v[e]);
-    } else if constexpr (R == 4) {
-      dft4(v[e][0], v[e][1], v[e][2], v[e][3]);
-      dft4(v[e][4], v[e][5], v[e][6], v[e][7]);
-    } else {
+  }
+  if constexpr (R == 8) {
+    dft8(v);
+  } else if constexpr (R == 4) {
+    dft4(v[0], v[1], v[2], v[3]);
+    dft4(v[4], v[5], v[6], v[7]);
+  } else {
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const float2 a0 = v[e][2 * r], a1 = v[e][2 * r + 1];
-        v[e][2 * r] = cadd(a0, a1);
-        v[e][2 * r + 1] = csub(a0, a1);
-      }
+    for (int r = 0; r < 4; ++r) {
+      const C2 a0 = v[2 * r], a1 = v[2 * r + 1];
+      v[2 * r] = cadd(a0, a1);
+      v[2 * r + 1] = csub(a0, a1);
     }
   }
-  __syncthreads();
-#pragma unroll
-  for (int e = 0; e < NB; ++e) {
-#pragma unroll
-    for (int r = 0; r < B; ++r) {
-      const int b = lt + r * (M / 8);
-      const int k = b & (Ns - 1);
-      const int base = (b - k) * R + k;
-#pragma unroll
-      for (int j = 0; j < R; ++j) zs[e][fe_pad(base + j * Ns)] = v[e][r * R + j];
-    }
-  }
-  __syncthreads();
 }
 
-// The equaliser in FP32, exactly: with |v| below vsat = ceil(7.5 2^21 / g)
-// the fix_36_24 product p = v g is an integer below 7.5 2^21 < 2^24, so
-// v (g 2^-21) is exact in FP32, and one fused multiply-add with 1.5 2^23
-// rounds it half to even; the sum's low four bits are the fix_4_3 code in
-// two's complement.  At or above vsat, |p| rounds to 8 or more and the code
-// saturates at +-7.
-__host__ __device__ inline float saturation_threshold(uint32_t g) {
-  return g == 0 ? 3.0e38f : (float)((15728640u + g - 1) / g);  // 7.5 2^21 = 15728640
+// A radix-8 pass in place: butterfly b writes its outputs to
+// (b div Ns) 8 Ns + (b mod Ns) + r Ns.  The first pass (Ns = 1) runs over the
+// whole unit, whose barrier separates its loads and stores and ends it; the
+// later ones run within the classes, the last one ended by the unit's barrier.
+template <int M, int NT, int NS, bool LAST, bool STW = false>
+__device__ __forceinline__ void fft_pass8(ulonglong2* z, int u, int lt, const float2 (&tw)[7],
+                                          const ulonglong2* stw = nullptr) {
+  constexpr int TPU = M / 8;
+  const int b = NS == 1 ? lt : class_butterfly<TPU>(lt);
+  C2 v[8];
+  butterflies<M, 8, STW>(v, z, {b}, NS, tw, stw);
+  if constexpr (NS == 1)
+    unit_sync<TPU, NT>(u);
+  else
+    class_sync<TPU>(lt);
+  const int k = b & (NS - 1);
+  const int to = (b - k) * 8 + k;
+  const int base = fe_pad(to);
+#pragma unroll
+  for (int j = 0; j < 8; ++j)  // (to is a multiple of 8 NS plus less than NS)
+    z_store(z, NS == 1 ? base + j : NS == 8 ? base + 9 * j : base + j * fe_pad(NS), v[j]);
+  if constexpr (NS == 1 || LAST)
+    unit_sync<TPU, NT>(u);
+  else
+    class_sync<TPU>(lt);
 }
-__device__ __forceinline__ int equalise_nibble(float vf, float gs, float vsat) {
-  const int code = __float_as_int(fmaf(vf, gs, 12582912.0f)) & 0xF;
-  return fabsf(vf) >= vsat ? (vf < 0.f ? 0x9 : 0x7) : code;
+
+// The equaliser in FP32, exactly: while the fix_36_24 product p = v g stays
+// below 7.5 2^21 < 2^24 in magnitude, v (g 2^-21) is exact in FP32, and one
+// fused multiply-add with 1.5 2^23 rounds it half to even; the sum's low four
+// bits are the fix_4_3 code in two's complement.  Larger products saturate at
+// +-7, which is the code of every v with p between 6.5 and 7.5 2^21: so the
+// spectra are clamped to +-w, an integer w near 7 2^21 / g, and to the 18-bit
+// range, before they are rounded to the code.  The interval is 14% of w wide,
+// so a thread keeps w as a bfloat16 (an integer: w >= 56), two to a register.
+__device__ __forceinline__ uint32_t clamp_bound(float gs) {  // gs = g 2^-21; bfloat16 bits
+  const float w = fminf(__fdividef(7.0f, gs), 200000.0f);    // (g = 0: infinity)
+  const float i = (w + 12582912.0f) - 12582912.0f;           // an integer
+  return (__float_as_uint(i) + 0x8000u) >> 16;
+}
+// The 18-bit range and w as one clamp: w below 2^17, else 2^17 - 0.75; with
+// kClampSkew the lower bound -(w + 0.375) rounds to -w or to -2^17.
+constexpr float kClampSkew = 0.375f;
+__device__ __forceinline__ float clamp18(uint32_t bits) {
+  return fminf(__uint_as_float(bits), 131071.25f);
 }
 
 // clamp(rne(x), -2^17, 2^17 - 1): clamping first keeps |x| < 2^22, where
 // adding 1.5 2^23 rounds x to the nearest integer, ties to even.  Returns
-// the sum; its low bits hold the integer, and subtracting 1.5 2^23 gives it
-// back exactly as a float.
-__device__ __forceinline__ float round18_biased(float x) {
+// the sum's bits less those of 1.5 2^23: the integer.
+__device__ __forceinline__ int round18(float x) {
   const float c = fminf(fmaxf(x, -131072.0f), 131071.0f);
-  return c + 12582912.0f;
+  return __float_as_int(c + 12582912.0f) - 0x4B400000;
 }
 
-// Byte r of w (biased: w holds x ^ 0x80 per byte, x the int8 sample) as the
-// float x, exactly: the byte becomes the low mantissa bits of 1.5 * 2^23,
-// and subtracting 1.5 * 2^23 + 128 leaves x (every step exact below 2^24).
-__device__ __forceinline__ float biased_byte_to_float(uint32_t w, int r) {
-  return __int_as_float((int)__byte_perm(w, 0x4B400000u, 0x7650u + (unsigned)r)) - 12583040.0f;
+// Bytes r and r + 1 of w (biased: w holds x ^ 0x80 per byte, x the int8 sample)
+// as the floats 1.5 2^23 + 128 + x: the byte becomes the low mantissa bits of
+// 1.5 2^23, and subtracting 1.5 2^23 + 128 leaves x (every step exact below 2^24).
+__device__ __forceinline__ uint64_t biased_bytes(uint32_t w, int r) {
+  return ((uint64_t)__byte_perm(w, 0x4B400000u, 0x7650u + (unsigned)(r + 1)) << 32) |
+         __byte_perm(w, 0x4B400000u, 0x7650u + (unsigned)r);
 }
 
-// Taps 0..3 of the filter for 8 consecutive samples of both inputs of a
-// pair, with aligned 8-byte rows: every tap's loads are issued before any
-// arithmetic (taps past `taps` load nothing and add nothing), then
-// y += h x in FP32 fused multiply-adds.
-__device__ __forceinline__ void fir_taps4(float (&y0)[8], float (&y1)[8], const float (&h)[4][8],
-                                          const int8_t* x0, const int8_t* x1, long long M,
-                                          int taps, bool has1) {
-  uint32_t w[4][4];
+constexpr float kByteBias = 12583040.0f;
+
+// Eight samples as pairs of floats, from the 8 bytes of an aligned load or one by one.
+__device__ __forceinline__ void samples8(uint64_t (&x)[4], int2 w) {
+  const uint32_t b[2] = {(uint32_t)w.x ^ 0x80808080u, (uint32_t)w.y ^ 0x80808080u};
+  const uint64_t bias = p_dup(kByteBias);
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    int2 a = make_int2(0, 0), b = make_int2(0, 0);
-    if (q < taps) {
-      a = __ldg(reinterpret_cast<const int2*>(x0 + q * M));
-      if (has1) b = __ldg(reinterpret_cast<const int2*>(x1 + q * M));
-    }
-    w[q][0] = (uint32_t)a.x ^ 0x80808080u;
-    w[q][1] = (uint32_t)a.y ^ 0x80808080u;
-    w[q][2] = (uint32_t)b.x ^ 0x80808080u;
-    w[q][3] = (uint32_t)b.y ^ 0x80808080u;
-  }
+  for (int r = 0; r < 4; ++r) x[r] = p_sub(biased_bytes(b[r >> 1], 2 * (r & 1)), bias);
+}
+__device__ __forceinline__ int2 load_bytes8(const int8_t* p) {
+  uint32_t w[2] = {0u, 0u};
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    if (q >= taps) break;
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      y0[r] = fmaf(h[q][r], biased_byte_to_float(w[q][r >> 2], r & 3), y0[r]);
-      y1[r] = fmaf(h[q][r], biased_byte_to_float(w[q][2 + (r >> 2)], r & 3), y1[r]);
-    }
-  }
+  for (int r = 0; r < 8; ++r) w[r >> 2] |= (uint32_t)(uint8_t)p[r] << (8 * (r & 3));
+  return make_int2((int)w[0], (int)w[1]);
 }
 
-// One tap of the filter for 8 consecutive samples of both inputs of a pair:
-// y += h x, in FP32 fused multiply-adds.
-__device__ __forceinline__ void fir_tap(float (&y0)[8], float (&y1)[8], const float (&h)[8],
-                                        const int8_t* x0, const int8_t* x1, bool has1, int vec_in) {
-  if (vec_in) {
-    const int2 w0 = __ldg(reinterpret_cast<const int2*>(x0));
-    const int2 w1 = has1 ? __ldg(reinterpret_cast<const int2*>(x1)) : make_int2(0, 0);
-    const uint32_t b0[2] = {(uint32_t)w0.x ^ 0x80808080u, (uint32_t)w0.y ^ 0x80808080u};
-    const uint32_t b1[2] = {(uint32_t)w1.x ^ 0x80808080u, (uint32_t)w1.y ^ 0x80808080u};
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      y0[r] = fmaf(h[r], biased_byte_to_float(b0[r >> 2], r & 3), y0[r]);
-      y1[r] = fmaf(h[r], biased_byte_to_float(b1[r >> 2], r & 3), y1[r]);
-    }
-  } else {
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      y0[r] = fmaf(h[r], (float)x0[r], y0[r]);
-      y1[r] = fmaf(h[r], has1 ? (float)x1[r] : 0.f, y1[r]);
-    }
-  }
-}
-
-// Two CTAs per SM where 256-thread CTAs fit twice (registers capped at 128,
-// with a few spills): measured 10% faster than one CTA at 217 registers.
+// Two CTAs per SM where 256-thread CTAs fit twice (registers capped at 128).
 __host__ __device__ constexpr int fe_min_blocks(int logm) { return logm <= 11 ? 2 : 1; }
 
-// POWER: accumulate Eq. 3's power sums (a separate instance, so that the
-// common launch without them keeps those registers free).
-template <int LOGM, bool POWER>
+// FE_FIGURES
+// POWER: accumulate Eq. 3's power sums.  FRAMED: at most four taps and
+// aligned frames, coefficients and frames in registers; otherwise any taps and
+// alignment.  (Instances of their own, so that each keeps the others'
+// registers free.)
+template <int LOGM, bool POWER, bool FRAMED>
 __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine_kernel(FeArgs a) {
   constexpr int M = 1 << LOGM, C = M / 2;
   constexpr int TPU = M / 8;                 // threads per FFT unit
@@ -286,235 +368,307 @@ __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine
   constexpr int P8 = LOGM / 3, REM = LOGM % 3;
   extern __shared__ __align__(16) uint8_t fe_smem[];
   const int tid = threadIdx.x, u = tid / TPU, lt = tid % TPU;
-  constexpr int kFeNB = fe_nb(LOGM);
-  float2* zs[kFeNB];
-#pragma unroll
-  for (int e = 0; e < kFeNB; ++e) zs[e] = reinterpret_cast<float2*>(fe_smem) + (e * U + u) * PM;
-  uint8_t* codes = fe_smem + (size_t)kFeNB * U * PM * sizeof(float2);  // [kFeGroup][C][2]
-  float2* ttab = reinterpret_cast<float2*>(codes + (size_t)C * 2 * kFeGroup);  // [Ns=8 | Ns=64][k][7]
+  ulonglong2* const z = reinterpret_cast<ulonglong2*>(fe_smem) + u * PM;
+  ulonglong2* const ttab = reinterpret_cast<ulonglong2*>(fe_smem) + U * PM;  // [Ns=8 | Ns=64][k][7]
+  // [channel of the thread][iteration][thread]: codes of two spectra, both inputs
+  uint32_t* const codes = reinterpret_cast<uint32_t*>(ttab + kTwTable) + tid;
+  // [channel of the thread][thread]: gains as g 2^-21 (exact) of the two inputs, and
+  // their clamp bounds, bfloat16 each (registers are what limits the CTA)
+  float2* const gains = reinterpret_cast<float2*>(codes - tid + 4 * kStageIts * NT) + tid;
+  uint32_t* const bounds = reinterpret_cast<uint32_t*>(gains - tid + 4 * NT) + tid;
   const int i0 = 2 * blockIdx.y;
   const bool has1 = i0 + 1 < a.n_inputs;
   const int N = a.n_inputs;
-  const int t0 = blockIdx.x * kFeGroup;
-  const int ng = min(kFeGroup, a.n_spectra - t0);
+  // this unit's spectra tu .. tu + per_unit - 1, two an iteration; the first
+  // unit's range, the earliest, says how many iterations the CTA makes
+  const int tu = (blockIdx.x * U + u) * a.per_unit;
+  const int n_it = (min(a.per_unit, a.n_spectra - (int)blockIdx.x * U * a.per_unit) + 1) / 2;
 
-  // per-thread constants: the filter taps of its 8 samples (up to 4 taps in
-  // registers) and the twiddles of every pass
-  float hr[4][8];
+  // per-thread constants: the filter taps of its 8 samples (neighbouring
+  // samples in pairs; absent taps are zeros) and the twiddles of every pass
+  uint64_t hr[4][4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    if (q < a.taps) {
-      const float4 hA = __ldg(reinterpret_cast<const float4*>(a.h + q * M + 8 * lt));
-      const float4 hB = __ldg(reinterpret_cast<const float4*>(a.h + q * M + 8 * lt + 4));
-      hr[q][0] = hA.x; hr[q][1] = hA.y; hr[q][2] = hA.z; hr[q][3] = hA.w;
-      hr[q][4] = hB.x; hr[q][5] = hB.y; hr[q][6] = hB.z; hr[q][7] = hB.w;
-    } else {
 #pragma unroll
-      for (int r = 0; r < 8; ++r) hr[q][r] = 0.f;
+    for (int r = 0; r < 4; r += 2) {
+      ulonglong2 v = make_ulonglong2(0, 0);
+      if (FRAMED && q < a.taps) v = __ldg(reinterpret_cast<const ulonglong2*>(a.h + q * M + 8 * lt + 2 * r));
+      hr[q][r] = v.x, hr[q][r + 1] = v.y;
     }
   }
   // passes at Ns = 8 and 64 read the shared table (filled here, first read
-  // after the filter's barrier); a pass at Ns = 512 (M = 4096) keeps registers
+  // after the barrier below); a pass at Ns = 512 (M = 4096) keeps registers
   for (int e = tid; e < kTwTable; e += NT) {
     const int big = e >= 56, q = big ? e - 56 : e, k = q / 7, j = q % 7 + 1;
     const int Ns = big ? 64 : 8;
-    if (M >= 8 * Ns) ttab[e] = __ldg(&a.w[j * k * (M / (8 * Ns))]);
+    if (M >= 8 * Ns) {
+      const float2 t = __ldg(&a.w[j * k * (M / (8 * Ns))]);
+      ttab[big ? 56 + tw64_row(k) * 7 + j - 1 : e] = make_ulonglong2(p_dup(t.x), p_dup(t.y));
+    }
   }
   float2 tw[1][7], twl[7];
-  if constexpr (P8 >= 4) load_twiddles<M, 8>(tw[0], lt, 512, a.w);
-  if constexpr (REM == 2) load_twiddles<M, 4>(twl, lt, 1 << (3 * P8), a.w);
-  if constexpr (REM == 1) load_twiddles<M, 2>(twl, lt, 1 << (3 * P8), a.w);
+  if constexpr (P8 >= 4) load_twiddles<M, 8>(tw[0], {class_butterfly<TPU>(lt)}, 512, a.w);
+  constexpr int RL = REM ? 1 << REM : 8;  // radix of the last pass
+  int bl[8 / RL] = {};                    // its butterflies, and the channels they give
+  if constexpr (REM != 0) {
+    last_butterflies<M, RL>(lt, bl);
+    load_twiddles<M, RL>(twl, bl, M / RL, a.w);
+  }
+  // channel k of this thread: the first RL/2 outputs of each butterfly
+  // (without a last pass of its own, lt + k TPU)
+  auto channel = [&](int k) { return REM ? bl[k / (RL / 2)] + k % (RL / 2) * (M / RL) : lt + k * TPU; };
 
-  float gs[4][2], vsat[4][2];  // gain as g 2^-21 (exact) and its saturation threshold
   unsigned long long pw[4][2];  // only used by the POWER instance
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    const int nu = lt + k * TPU;
+    const long long g = (long long)channel(k) * N + i0;
+    const float g0 = (float)a.gain[g] * 4.76837158203125e-07f;  // 2^-21
+    const float g1 = has1 ? (float)a.gain[g + 1] * 4.76837158203125e-07f : 0.f;
+    gains[k * NT] = make_float2(g0, g1);
+    bounds[k * NT] = clamp_bound(g0) | (clamp_bound(g1) << 16);
+    pw[k][0] = pw[k][1] = 0ull;
+  }
+  __syncthreads();  // the table
+
+  const int8_t* const xt = a.adc + (long long)i0 * a.adc_stride + (long long)tu * M + 8 * lt;
+  // the five frames of the unit's next two spectra, both inputs, as loaded:
+  // requested an iteration ahead, so that the FFT hides their latency (loads
+  // at the filter itself, with the L1 prefetched, cost 18%)
+  int2 raw[5][2];
+  auto load_frame = [&](int f, int s) {  // frame f of spectra s, s + 1 (if one of them uses it)
+    raw[f][0] = raw[f][1] = make_int2(0, 0);
+    if (f > min(2, a.n_spectra - tu - s) + a.taps - 2) return;
+    const int8_t* x = xt + (long long)(s + f) * M;
+    raw[f][0] = __ldg(reinterpret_cast<const int2*>(x));
+    if (has1) raw[f][1] = __ldg(reinterpret_cast<const int2*>(x + a.adc_stride));
+  };
+  if constexpr (FRAMED) {
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const uint32_t gj = (j == 0 || has1) ? a.gain[(long long)nu * N + i0 + j] : 0u;
-      gs[k][j] = (float)gj * 4.76837158203125e-07f;  // 2^-21
-      vsat[k][j] = saturation_threshold(gj);
-      pw[k][j] = 0ull;
-    }
+    for (int f = 0; f < 5; ++f) load_frame(f, 0);
   }
 
-  for (int sb = 0; sb < ng; sb += kFeNB * U) {
+  for (int it = 0; it < n_it; ++it) {
+    const int s = 2 * it;                              // this unit's spectra: tu + s and the next
+    const int n_act = min(2, a.n_spectra - tu - s);    // how many of them exist (<= 0: none)
     // ---- polyphase filter: y[n] = sum_q h[q M + n] x[(t + q) M + n]
-    if (U == 1 && a.vec_in && a.taps <= 4) {
-      // One unit per CTA: the unit's spectra sb, sb + 1, ... are adjacent and
-      // share frames, so each frame is loaded and converted once and added
-      // into every spectrum that uses it (static tap indices).
-      constexpr int NF = kFeNB + 3;  // frames of kFeNB spectra at up to 4 taps
-      const int8_t* xb = a.adc + (long long)i0 * a.adc_stride + (long long)(t0 + sb) * M + 8 * lt;
-      const int last = min(ng - 1 - sb, kFeNB - 1);  // last active spectrum of the iteration
-      float y[kFeNB][2][8];
+    // The two spectra share frames: each is converted once and added into the
+    // spectra that use it, in the order of their taps.  Pairs here are
+    // neighbouring samples, as the coefficients lie.
+    uint64_t y[2][2][4];  // [spectrum][input][sample pair]
 #pragma unroll
-      for (int e = 0; e < kFeNB; ++e)
+    for (int e = 0; e < 2; ++e)
 #pragma unroll
-        for (int r = 0; r < 8; ++r) y[e][0][r] = y[e][1][r] = 0.f;
+      for (int r = 0; r < 4; ++r) y[e][0][r] = y[e][1][r] = 0ull;
+    if constexpr (FRAMED) {
 #pragma unroll
-      for (int f = 0; f < NF; ++f) {
-        if (f > last + a.taps - 1) break;  // frames past the last active spectrum's taps
-        const int2 w0 = __ldg(reinterpret_cast<const int2*>(xb + (long long)f * M));
-        const int2 w1 = has1 ? __ldg(reinterpret_cast<const int2*>(xb + a.adc_stride + (long long)f * M))
-                             : make_int2(0, 0);
-        const uint32_t b[4] = {(uint32_t)w0.x ^ 0x80808080u, (uint32_t)w0.y ^ 0x80808080u,
-                               (uint32_t)w1.x ^ 0x80808080u, (uint32_t)w1.y ^ 0x80808080u};
-        float x[2][8];
+      for (int f = 0; f < 5; ++f) {
+        if (f > a.taps) break;
+        uint64_t x[2][4];  // (frames past the last spectrum's are zeros)
+        samples8(x[0], raw[f][0]);
+        samples8(x[1], raw[f][1]);
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-          x[0][r] = biased_byte_to_float(b[r >> 2], r & 3);
-          x[1][r] = biased_byte_to_float(b[2 + (r >> 2)], r & 3);
-        }
-#pragma unroll
-        for (int e = 0; e < kFeNB; ++e) {
+        for (int e = 0; e < 2; ++e) {
           const int q = f - e;  // this frame is tap q of spectrum e
-          if (q < 0 || q > 3 || q >= a.taps || e > last) continue;
+          if (q < 0 || q > 3) continue;
 #pragma unroll
-          for (int r = 0; r < 8; ++r) {
-            y[e][0][r] = fmaf(hr[q][r], x[0][r], y[e][0][r]);
-            y[e][1][r] = fmaf(hr[q][r], x[1][r], y[e][1][r]);
+          for (int r = 0; r < 4; ++r) {
+            y[e][0][r] = p_fma(hr[q][r], x[0][r], y[e][0][r]);
+            y[e][1][r] = p_fma(hr[q][r], x[1][r], y[e][1][r]);
           }
         }
       }
+      // the next iteration's frames: two spectra on, taps - 1 of the five stay
+      if (it + 1 < n_it) {
 #pragma unroll
-      for (int e = 0; e < kFeNB; ++e) {
-#pragma unroll
-        for (int r = 0; r < 8; ++r) zs[e][fe_pad(8 * lt + r)] = make_float2(y[e][0][r], y[e][1][r]);
-      }
-      // the next iteration's newest frames come from DRAM: ask for those of
-      // its active spectra now
-#pragma unroll
-      for (int e = 0; e < kFeNB; ++e) {
-        if (sb + kFeNB + e >= ng) break;
-        const int8_t* nx = xb + (long long)(kFeNB + e + a.taps - 1) * M;
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(nx));
-        if (has1) asm volatile("prefetch.global.L1 [%0];" ::"l"(nx + a.adc_stride));
-      }
-    } else {
-#pragma unroll
-    for (int e = 0; e < kFeNB; ++e) {
-      const int s = sb + e * U + u;
-      const bool active = s < ng;
-      const long long t = t0 + s;
-      float y0[8], y1[8];
-#pragma unroll
-      for (int r = 0; r < 8; ++r) y0[r] = y1[r] = 0.f;
-      if (active) {
-        const int8_t* x0 = a.adc + (long long)i0 * a.adc_stride + t * M + 8 * lt;
-        const int8_t* x1 = x0 + a.adc_stride;
-        // taps 0..3 with their coefficients in registers (static indices),
-        // then any further taps with coefficients from the table
-        if (a.vec_in) {
-          fir_taps4(y0, y1, hr, x0, x1, M, a.taps, has1);
-        } else {
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (q < a.taps)
-              fir_tap(y0, y1, hr[q], x0 + (long long)q * M, x1 + (long long)q * M, has1, 0);
-        }
-        for (int q = 4; q < a.taps; ++q) {
-          float hq[8];
-          const float4 hA = __ldg(reinterpret_cast<const float4*>(a.h + q * M + 8 * lt));
-          const float4 hB = __ldg(reinterpret_cast<const float4*>(a.h + q * M + 8 * lt + 4));
-          hq[0] = hA.x; hq[1] = hA.y; hq[2] = hA.z; hq[3] = hA.w;
-          hq[4] = hB.x; hq[5] = hB.y; hq[6] = hB.z; hq[7] = hB.w;
-          fir_tap(y0, y1, hq, x0 + (long long)q * M, x1 + (long long)q * M, has1, a.vec_in);
+        for (int f = 0; f < 5; ++f) {
+          if (f < 3 && f <= a.taps - 2)
+            raw[f][0] = raw[f + 2][0], raw[f][1] = raw[f + 2][1];
+          else
+            load_frame(f, s + 2);
         }
       }
+    } else {  // any number of taps, any alignment
+      uint64_t hp[4] = {0ull, 0ull, 0ull, 0ull};  // the tap before
+      for (int f = 0; f < n_act + a.taps - 1; ++f) {
+        const int8_t* xf = xt + (long long)(s + f) * M;
+        uint64_t x[2][4], hq[4] = {0ull, 0ull, 0ull, 0ull};
+        if (f < a.taps) {
+          const ulonglong2 hA = __ldg(reinterpret_cast<const ulonglong2*>(a.h + f * M + 8 * lt));
+          const ulonglong2 hB = __ldg(reinterpret_cast<const ulonglong2*>(a.h + f * M + 8 * lt + 4));
+          hq[0] = hA.x, hq[1] = hA.y, hq[2] = hB.x, hq[3] = hB.y;
+        }
+        samples8(x[0], a.vec_in ? __ldg(reinterpret_cast<const int2*>(xf)) : load_bytes8(xf));
+        xf += a.adc_stride;
+        samples8(x[1], !has1 ? make_int2(0, 0)
+                             : a.vec_in ? __ldg(reinterpret_cast<const int2*>(xf)) : load_bytes8(xf));
 #pragma unroll
-      for (int r = 0; r < 8; ++r) zs[e][fe_pad(8 * lt + r)] = make_float2(y0[r], y1[r]);
-      // the next iteration's newest frame comes from DRAM: ask for it now
-      if (active && s + kFeNB * U < ng) {
-        const int8_t* nx =
-            a.adc + (long long)i0 * a.adc_stride + (t + kFeNB * U + a.taps - 1) * M + 8 * lt;
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(nx));
-        if (has1) asm volatile("prefetch.global.L1 [%0];" ::"l"(nx + a.adc_stride));
+        for (int r = 0; r < 4; ++r) {
+          if (f < a.taps) {
+            y[0][0][r] = p_fma(hq[r], x[0][r], y[0][0][r]);
+            y[0][1][r] = p_fma(hq[r], x[1][r], y[0][1][r]);
+          }
+          if (f > 0 && n_act > 1) {
+            y[1][0][r] = p_fma(hp[r], x[0][r], y[1][0][r]);
+            y[1][1][r] = p_fma(hp[r], x[1][r], y[1][1][r]);
+          }
+          hp[r] = hq[r];
+        }
       }
     }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      float v[2][2][2];  // [spectrum][input][sample]
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) p_unpack(y[e][j][r], v[e][j][0], v[e][j][1]);
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        z_store(z, fe_pad(8 * lt) + 2 * r + i, {p_pack(v[0][0][i], v[1][0][i]), p_pack(v[0][1][i], v[1][1][i])});
     }
-    __syncthreads();
-    // ---- FFTs of y_2k + j y_2k+1 (natural order out), kFeNB side by side
-    fft_pass<M, 8, kFeNB>(zs, lt, 1, twl);  // first pass: no twiddles
-    if constexpr (P8 >= 2) fft_pass<M, 8, kFeNB, true>(zs, lt, 8, twl, ttab);
-    if constexpr (P8 >= 3) fft_pass<M, 8, kFeNB, true>(zs, lt, 64, twl, ttab + 56);
-    if constexpr (P8 >= 4) fft_pass<M, 8, kFeNB>(zs, lt, 512, tw[0]);
-    if constexpr (REM == 2) fft_pass<M, 4, kFeNB>(zs, lt, 1 << (3 * P8), twl);
-    if constexpr (REM == 1) fft_pass<M, 2, kFeNB>(zs, lt, 1 << (3 * P8), twl);
+    unit_sync<TPU, NT>(u);
+    // ---- FFTs of y_2k + j y_2k+1 (natural order out)
+    fft_pass8<M, NT, 1, P8 == 1>(z, u, lt, twl);  // first pass: no twiddles
+    if constexpr (P8 >= 2) fft_pass8<M, NT, 8, P8 == 2, true>(z, u, lt, twl, ttab);
+    if constexpr (P8 >= 3) fft_pass8<M, NT, 64, P8 == 3, true>(z, u, lt, twl, ttab + 56);
+    if constexpr (P8 >= 4) fft_pass8<M, NT, 512, P8 == 4>(z, u, lt, tw[0]);
+    C2 v[8];
+    if constexpr (REM != 0) butterflies<M, RL>(v, z, bl, M / RL, twl);
     // ---- Eq. 2 separation, 18-bit rounding, equaliser
-#pragma unroll
-    for (int e = 0; e < kFeNB; ++e) {
-      const int s = sb + e * U + u;
-      if (s >= ng) continue;
-      const long long t = t0 + s;
-      const float2* z = zs[e];
+    if (n_act > 0) {
+      const uint64_t scale = p_dup(a.scale), magic = p_dup(12582912.0f);
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const int nu = lt + k * TPU;
-        const float2 zp = z[fe_pad(nu)], zm = z[fe_pad((M - nu) & (M - 1))];
-        const float X[2][2] = {{(zp.x + zm.x) * a.scale, (zp.y - zm.y) * a.scale},
-                               {(zp.y + zm.y) * a.scale, (zm.x - zp.x) * a.scale}};
-        uint32_t pair = 0;  // the codes of inputs i0 and i0 + 1: one 16-bit store
+        const int nu = channel(k);
+        C2 zp, zm;
+        if constexpr (REM != 0) {
+          constexpr int H = RL / 2;
+          const int q = k / H, r = k % H;  // output r of butterfly q; its mirror is output RL-1-r of butterfly q^1
+          zp = v[q * RL + r];
+          zm = v[(q ^ 1) * RL + RL - 1 - r];
+          if (q < 2 && lt == 0) zm = q == 0 ? v[(RL - r) % RL] : v[RL + RL - 1 - r];  // its own mirror
+        } else {
+          zp = z_load(z, fe_pad(nu));
+          zm = z_load(z, fe_pad((M - nu) & (M - 1)));
+        }
+        // X[input][re, im] of both spectra
+        const uint64_t X[2][2] = {{p_mul(p_add(zp.x, zm.x), scale), p_mul(p_sub(zp.y, zm.y), scale)},
+                                  {p_mul(p_add(zp.y, zm.y), scale), p_mul(p_sub(zm.x, zp.x), scale)}};
+        if (a.spec || a.v18) {
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            if (j == 1 && !has1) break;
+            float xr[2], xi[2];
+            p_unpack(X[j][0], xr[0], xr[1]);
+            p_unpack(X[j][1], xi[0], xi[1]);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              if (e >= n_act) break;
+              const long long ei = (((long long)(tu + s + e) * C + nu) * N + i0 + j) * 2;
+              if (a.spec) *reinterpret_cast<float2*>(a.spec + ei) = make_float2(xr[e], xi[e]);
+              if (a.v18) *reinterpret_cast<int2*>(a.v18 + ei) = make_int2(round18(xr[e]), round18(xi[e]));
+            }
+          }
+        }
+        const float2 gk = gains[k * NT];
+        const uint32_t bound = bounds[k * NT];
+        uint32_t q[2][2][2];  // [re, im][input][spectrum], the code in the low four bits
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-          if (j == 1 && !has1) break;
-          const float sr = round18_biased(X[j][0]), si = round18_biased(X[j][1]);
-          const int vr = __float_as_int(sr) - 0x4B400000, vi = __float_as_int(si) - 0x4B400000;
-          if (a.spec || a.v18) {
-            const long long ei = ((t * C + nu) * N + i0 + j) * 2;
-            if (a.spec) *reinterpret_cast<float2*>(a.spec + ei) = make_float2(X[j][0], X[j][1]);
-            if (a.v18) *reinterpret_cast<int2*>(a.v18 + ei) = make_int2(vr, vi);
+          const uint64_t g = p_dup(j ? gk.y : gk.x);
+          const uint32_t wb = j ? bound & 0xFFFF0000u : bound << 16;
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            float x0, x1;
+            p_unpack(X[j][c], x0, x1);
+            uint64_t f;  // the rounded spectrum, clamped to the bound
+            if constexpr (POWER) {  // the 18-bit value first, for the sums
+              const uint64_t v18 = p_add(p_pack(fminf(fmaxf(x0, -131072.0f), 131071.0f),
+                                                fminf(fmaxf(x1, -131072.0f), 131071.0f)), magic);
+              const int i0v = (int)(uint32_t)v18 - 0x4B400000, i1v = (int)(uint32_t)(v18 >> 32) - 0x4B400000;
+              pw[k][j] += (unsigned long long)((long long)i0v * i0v);
+              if (n_act > 1) pw[k][j] += (unsigned long long)((long long)i1v * i1v);
+              p_unpack(p_sub(v18, magic), x0, x1);
+              const float w = __uint_as_float(wb);
+              f = p_pack(fminf(fmaxf(x0, -w), w), fminf(fmaxf(x1, -w), w));
+            } else {
+              const float hi = clamp18(wb), lo = -(hi + kClampSkew);
+              f = p_sub(p_add(p_pack(fminf(fmaxf(x0, lo), hi), fminf(fmaxf(x1, lo), hi)), magic), magic);
+            }
+            const uint64_t e = p_fma(f, g, magic);
+            q[c][j][0] = (uint32_t)e;
+            q[c][j][1] = (uint32_t)(e >> 32);
           }
-          if constexpr (POWER) pw[k][j] += (unsigned long long)((long long)vr * vr + (long long)vi * vi);
-          const int qr = equalise_nibble(sr - 12582912.0f, gs[k][j], vsat[k][j]);
-          const int qi = equalise_nibble(si - 12582912.0f, gs[k][j], vsat[k][j]);
-          pair |= (uint32_t)(a.lo_is_real ? (qi << 4) | qr : (qr << 4) | qi) << (8 * j);
         }
-        *reinterpret_cast<uint16_t*>(codes + (s * C + nu) * 2) = (uint16_t)pair;
+        // bytes [spectrum][input] of the real and the imaginary codes, then both nibbles
+        uint32_t nib[2];
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+          nib[c] = __byte_perm(__byte_perm(q[c][0][0], q[c][1][0], 0x0040), __byte_perm(q[c][0][1], q[c][1][1], 0x0040), 0x5410);
+        const uint32_t up = a.lo_is_real ? nib[1] : nib[0], down = a.lo_is_real ? nib[0] : nib[1];
+        const uint32_t word = ((up << 4) & 0xF0F0F0F0u) | (down & 0x0F0F0F0Fu);
+        if (a.layout == CORR_L_CIT) {
+          codes[(k * kStageIts + it % kStageIts) * NT] = word;
+        } else if (a.out) {  // [t][c][i]
+          uint8_t* o = a.out + ((long long)(tu + s) * C + nu) * N + i0;
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            if (e >= n_act) break;
+            o[(long long)e * C * N] = (uint8_t)(word >> (16 * e));
+            if (has1) o[(long long)e * C * N + 1] = (uint8_t)(word >> (16 * e + 8));
+          }
+        }
       }
     }
-    __syncthreads();
+    // ---- codes out to [c][i][t], when a stage is full: the thread's own
+    // channels, 16 spectra (or all it has, fewer) of each input as one piece
+    if (a.out && a.layout == CORR_L_CIT && (it % kStageIts == kStageIts - 1 || it == n_it - 1)) {
+      const int first = it / kStageIts * kStageIts;  // iteration of the stage's first spectra
+      const int cnt = min(2 * (it + 1 - first), a.n_spectra - tu - 2 * first);
+      const int whole = min(a.per_unit, 2 * kStageIts);
+#pragma unroll 1
+      for (int k = 0; k < 4 && cnt > 0; ++k) {
+        int nu = channel(0);  // (a dynamic k)
+#pragma unroll
+        for (int kk = 1; kk < 4; ++kk)
+          if (kk == k) nu = channel(kk);
+        const uint32_t* const src = codes + k * kStageIts * NT;
+        uint8_t* o = a.out + ((long long)nu * N + i0) * a.out_stride + tu + 2 * first;
+        if (a.vec_out && cnt == whole && whole >= 4) {
+          uint32_t w[2][4];
+#pragma unroll
+          for (int h = 0; h < 4; ++h) {
+            const uint32_t w0 = 4 * h < cnt ? src[2 * h * NT] : 0u, w1 = 4 * h < cnt ? src[(2 * h + 1) * NT] : 0u;
+            w[0][h] = __byte_perm(w0, w1, 0x6420);
+            w[1][h] = __byte_perm(w0, w1, 0x7531);
+          }
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            if (j == 1 && !has1) break;
+            uint8_t* d = o + j * a.out_stride;
+            if (whole == 16)
+              *reinterpret_cast<uint4*>(d) = make_uint4(w[j][0], w[j][1], w[j][2], w[j][3]);
+            else if (whole == 8)
+              *reinterpret_cast<uint2*>(d) = make_uint2(w[j][0], w[j][1]);
+            else
+              *reinterpret_cast<uint32_t*>(d) = w[j][0];
+          }
+        } else {
+          for (int q = 0; q < cnt; ++q) {
+            const uint32_t w = src[(q >> 1) * NT] >> (16 * (q & 1));
+            o[q] = (uint8_t)w;
+            if (has1) o[a.out_stride + q] = (uint8_t)(w >> 8);
+          }
+        }
+      }
+    }
+    unit_sync<TPU, NT>(u);  // z is read: the next iteration may fill it
   }
 
-  // ---- codes out.  Staging is [spectrum][channel][input], so a thread
-  // gathers one (channel, input) row of 32 spectra with conflict-free byte
-  // loads (consecutive threads, consecutive rows) and stores it as two
-  // 16-byte pieces of the [c][i][t] output.
-  const int nj = has1 ? 2 : 1;
-  if (a.out) {
-    if (a.layout == CORR_L_CIT) {
-      for (int row = tid; row < 2 * C; row += NT) {
-        const int nu = row >> 1, j = row & 1;
-        if (j >= nj) continue;
-        uint8_t* o = a.out + ((long long)nu * N + i0 + j) * a.out_stride + t0;
-        if (a.vec_out && ng == kFeGroup) {
-          uint32_t wv[8];
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            wv[q] = (uint32_t)codes[(4 * q) * 2 * C + row] |
-                    ((uint32_t)codes[(4 * q + 1) * 2 * C + row] << 8) |
-                    ((uint32_t)codes[(4 * q + 2) * 2 * C + row] << 16) |
-                    ((uint32_t)codes[(4 * q + 3) * 2 * C + row] << 24);
-          *reinterpret_cast<uint4*>(o) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-          *reinterpret_cast<uint4*>(o + 16) = make_uint4(wv[4], wv[5], wv[6], wv[7]);
-        } else {
-          for (int s = 0; s < ng; ++s) o[s] = codes[s * 2 * C + row];
-        }
-      }
-    } else {  // [t][c][i]
-      for (int e = tid; e < ng * C; e += NT) {
-        const int s = e / C, nu = e - s * C;
-        uint8_t* o = a.out + ((long long)(t0 + s) * C + nu) * N + i0;
-        o[0] = codes[(s * C + nu) * 2];
-        if (has1) o[1] = codes[(s * C + nu) * 2 + 1];
-      }
-    }
-  }
   if constexpr (POWER) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const int nu = lt + k * TPU;
+      const int nu = channel(k);
       // every unit of the CTA summed its own spectra: add them all
       atomicAdd(a.power + (long long)nu * N + i0, pw[k][0]);
       if (has1) atomicAdd(a.power + (long long)nu * N + i0 + 1, pw[k][1]);
@@ -522,24 +676,35 @@ __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine
   }
 }
 
-template <int LOGM, bool POWER>
+template <int LOGM, bool POWER, bool FRAMED>
 cudaError_t fe_launch_one(const FeArgs& a, int n_pairs, cudaStream_t s) {
   constexpr size_t smem = fe_smem_bytes<LOGM>();
   static bool attr = false;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(fengine_kernel<LOGM, POWER>,
+    cudaError_t e = cudaFuncSetAttribute(fengine_kernel<LOGM, POWER, FRAMED>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  const dim3 grid((a.n_spectra + kFeGroup - 1) / kFeGroup, n_pairs);
-  fengine_kernel<LOGM, POWER><<<grid, fe_threads(LOGM), smem, s>>>(a);
+  // Spectra per unit: 32 (few prologues, the 16-spectra pieces of the output
+  // whole), or fewer while that leaves slots of the chip idle.
+  FeArgs b = a;
+  const int slots = device_sm_count() * fe_min_blocks(LOGM);
+  for (b.per_unit = 32; b.per_unit > 2; b.per_unit /= 2) {
+    const int group = b.per_unit * fe_units(LOGM);
+    if ((long long)((a.n_spectra + group - 1) / group) * n_pairs >= 2 * slots) break;
+  }
+  const int group = b.per_unit * fe_units(LOGM);
+  const dim3 grid((a.n_spectra + group - 1) / group, n_pairs);
+  fengine_kernel<LOGM, POWER, FRAMED><<<grid, fe_threads(LOGM), smem, s>>>(b);
   return cudaGetLastError();
 }
 
 template <int LOGM>
 cudaError_t fe_launch(const FeArgs& a, int n_pairs, cudaStream_t s) {
-  return a.power ? fe_launch_one<LOGM, true>(a, n_pairs, s) : fe_launch_one<LOGM, false>(a, n_pairs, s);
+  if (a.vec_in && a.taps <= 4)
+    return a.power ? fe_launch_one<LOGM, true, true>(a, n_pairs, s) : fe_launch_one<LOGM, false, true>(a, n_pairs, s);
+  return a.power ? fe_launch_one<LOGM, true, false>(a, n_pairs, s) : fe_launch_one<LOGM, false, false>(a, n_pairs, s);
 }
 
 bool fe_is_device(const void* p) {
