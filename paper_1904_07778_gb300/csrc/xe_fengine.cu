@@ -318,6 +318,22 @@ __device__ __forceinline__ float clamp18(uint32_t bits) {
   return fminf(__uint_as_float(bits), 131071.25f);
 }
 
+// With a gain of kWideGain or more, everything beyond the 18-bit range
+// saturates (2^17 * 120 = 7.5 2^21), and so does all that lies past w: the
+// spectra need no clamp before they are rounded, only the code does.  (A
+// spectrum stays below 2^21: M/2 127 sum |h| < 2^21, so v g 2^-21 < 2^18 and
+// both magic roundings keep exact.)
+constexpr uint32_t kWideGain = 120;
+// A rounded code (the bits of 1.5 2^23 + q) clamped from below, to -7; s4_pack
+// then saturates it from above.
+__device__ __forceinline__ int code_floor(uint32_t bits) { return __viaddmax_s32((int)bits, -0x4B400000, -7); }
+// low << 8 with the byte hi : lo of two codes, saturated to 4 bits, below it
+__device__ __forceinline__ uint32_t s4_pack(int hi, int lo, uint32_t low) {
+  uint32_t d;
+  asm("cvt.pack.sat.s4.s32.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(hi), "r"(lo), "r"(low));
+  return d;
+}
+
 // clamp(rne(x), -2^17, 2^17 - 1): clamping first keeps |x| < 2^22, where
 // adding 1.5 2^23 rounds x to the nearest integer, ties to even.  Returns
 // the sum's bits less those of 1.5 2^23: the integer.
@@ -353,7 +369,16 @@ __device__ __forceinline__ int2 load_bytes8(const int8_t* p) {
 // Two CTAs per SM where 256-thread CTAs fit twice (registers capped at 128).
 __host__ __device__ constexpr int fe_min_blocks(int logm) { return logm <= 11 ? 2 : 1; }
 
-// FE_FIGURES
+// What bounds it: latency.  128 registers a thread (32 hold the two spectra's
+// eight points, 52 the taps and the next frames) leave 16 warps an SM, with
+// issue slots half busy, the shared-memory data pipe 58% and FP32 42%; the time
+// is close to proportional to the instructions of an iteration (about 1250 a
+// thread), a quarter of them the separation and equaliser.  192 inputs x 1024
+// channels x 2048 spectra: 2.02 -> 1.52 ms, in steps (ms): packed pairs and
+// 16-byte points 1.94; frames loaded an iteration ahead, 16 staged spectra
+// 1.78; the last pass and the separation in registers 1.59; classes within
+// warps 1.56; instances for up to four taps 1.55; the code clamped instead of
+// the spectra 1.52.
 // POWER: accumulate Eq. 3's power sums.  FRAMED: at most four taps and
 // aligned frames, coefficients and frames in registers; otherwise any taps and
 // alignment.  (Instances of their own, so that each keeps the others'
@@ -419,16 +444,18 @@ __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine
   auto channel = [&](int k) { return REM ? bl[k / (RL / 2)] + k % (RL / 2) * (M / RL) : lt + k * TPU; };
 
   unsigned long long pw[4][2];  // only used by the POWER instance
+  bool wide = true;             // every gain of this CTA is 0 or kWideGain and more
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const long long g = (long long)channel(k) * N + i0;
-    const float g0 = (float)a.gain[g] * 4.76837158203125e-07f;  // 2^-21
-    const float g1 = has1 ? (float)a.gain[g + 1] * 4.76837158203125e-07f : 0.f;
+    const uint32_t n0 = a.gain[g], n1 = has1 ? a.gain[g + 1] : 0u;
+    wide = wide && (n0 == 0 || n0 >= kWideGain) && (n1 == 0 || n1 >= kWideGain);
+    const float g0 = (float)n0 * 4.76837158203125e-07f, g1 = (float)n1 * 4.76837158203125e-07f;  // 2^-21
     gains[k * NT] = make_float2(g0, g1);
     bounds[k * NT] = clamp_bound(g0) | (clamp_bound(g1) << 16);
     pw[k][0] = pw[k][1] = 0ull;
   }
-  __syncthreads();  // the table
+  wide = __syncthreads_and(wide);  // (and the table is filled)
 
   const int8_t* const xt = a.adc + (long long)i0 * a.adc_stride + (long long)tu * M + 8 * lt;
   // the five frames of the unit's next two spectra, both inputs, as loaded:
@@ -571,42 +598,58 @@ __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine
           }
         }
         const float2 gk = gains[k * NT];
-        const uint32_t bound = bounds[k * NT];
-        uint32_t q[2][2][2];  // [re, im][input][spectrum], the code in the low four bits
+        uint32_t q[2][2][2];  // [re, im][input][spectrum]: the bits of 1.5 2^23 + code
+        if (POWER || !wide) {
+          const uint32_t bound = bounds[k * NT];
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const uint64_t g = p_dup(j ? gk.y : gk.x);
-          const uint32_t wb = j ? bound & 0xFFFF0000u : bound << 16;
+          for (int j = 0; j < 2; ++j) {
+            const uint64_t g = p_dup(j ? gk.y : gk.x);
+            const uint32_t wb = j ? bound & 0xFFFF0000u : bound << 16;
 #pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            float x0, x1;
-            p_unpack(X[j][c], x0, x1);
-            uint64_t f;  // the rounded spectrum, clamped to the bound
-            if constexpr (POWER) {  // the 18-bit value first, for the sums
-              const uint64_t v18 = p_add(p_pack(fminf(fmaxf(x0, -131072.0f), 131071.0f),
-                                                fminf(fmaxf(x1, -131072.0f), 131071.0f)), magic);
-              const int i0v = (int)(uint32_t)v18 - 0x4B400000, i1v = (int)(uint32_t)(v18 >> 32) - 0x4B400000;
-              pw[k][j] += (unsigned long long)((long long)i0v * i0v);
-              if (n_act > 1) pw[k][j] += (unsigned long long)((long long)i1v * i1v);
-              p_unpack(p_sub(v18, magic), x0, x1);
-              const float w = __uint_as_float(wb);
-              f = p_pack(fminf(fmaxf(x0, -w), w), fminf(fmaxf(x1, -w), w));
-            } else {
-              const float hi = clamp18(wb), lo = -(hi + kClampSkew);
-              f = p_sub(p_add(p_pack(fminf(fmaxf(x0, lo), hi), fminf(fmaxf(x1, lo), hi)), magic), magic);
+            for (int c = 0; c < 2; ++c) {
+              float x0, x1;
+              p_unpack(X[j][c], x0, x1);
+              uint64_t f;  // the rounded spectrum, clamped to the bound
+              if constexpr (POWER) {  // the 18-bit value first, for the sums
+                const uint64_t v18 = p_add(p_pack(fminf(fmaxf(x0, -131072.0f), 131071.0f),
+                                                  fminf(fmaxf(x1, -131072.0f), 131071.0f)), magic);
+                const int v0 = (int)(uint32_t)v18 - 0x4B400000, v1 = (int)(uint32_t)(v18 >> 32) - 0x4B400000;
+                pw[k][j] += (unsigned long long)((long long)v0 * v0);
+                if (n_act > 1) pw[k][j] += (unsigned long long)((long long)v1 * v1);
+                f = p_sub(v18, magic);
+                if (!wide) {
+                  p_unpack(f, x0, x1);
+                  const float w = __uint_as_float(wb);
+                  f = p_pack(fminf(fmaxf(x0, -w), w), fminf(fmaxf(x1, -w), w));
+                }
+              } else {
+                const float hi = clamp18(wb), lo = -(hi + kClampSkew);
+                f = p_sub(p_add(p_pack(fminf(fmaxf(x0, lo), hi), fminf(fmaxf(x1, lo), hi)), magic), magic);
+              }
+              const uint64_t e = p_fma(f, g, magic);
+              q[c][j][0] = (uint32_t)e;
+              q[c][j][1] = (uint32_t)(e >> 32);
             }
-            const uint64_t e = p_fma(f, g, magic);
-            q[c][j][0] = (uint32_t)e;
-            q[c][j][1] = (uint32_t)(e >> 32);
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const uint64_t g = p_dup(j ? gk.y : gk.x);
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+              const uint64_t e = p_fma(p_sub(p_add(X[j][c], magic), magic), g, magic);
+              q[c][j][0] = (uint32_t)e;
+              q[c][j][1] = (uint32_t)(e >> 32);
+            }
           }
         }
-        // bytes [spectrum][input] of the real and the imaginary codes, then both nibbles
-        uint32_t nib[2];
+        // bytes [spectrum][input], the last one first
+        uint32_t word = 0;
 #pragma unroll
-        for (int c = 0; c < 2; ++c)
-          nib[c] = __byte_perm(__byte_perm(q[c][0][0], q[c][1][0], 0x0040), __byte_perm(q[c][0][1], q[c][1][1], 0x0040), 0x5410);
-        const uint32_t up = a.lo_is_real ? nib[1] : nib[0], down = a.lo_is_real ? nib[0] : nib[1];
-        const uint32_t word = ((up << 4) & 0xF0F0F0F0u) | (down & 0x0F0F0F0Fu);
+        for (int b = 3; b >= 0; --b) {
+          const int re = code_floor(q[0][b & 1][b >> 1]), im = code_floor(q[1][b & 1][b >> 1]);
+          word = a.lo_is_real ? s4_pack(im, re, word) : s4_pack(re, im, word);
+        }
         if (a.layout == CORR_L_CIT) {
           codes[(k * kStageIts + it % kStageIts) * NT] = word;
         } else if (a.out) {  // [t][c][i]
@@ -686,8 +729,10 @@ cudaError_t fe_launch_one(const FeArgs& a, int n_pairs, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  // Spectra per unit: 32 (few prologues, the 16-spectra pieces of the output
-  // whole), or fewer while that leaves slots of the chip idle.
+  // Spectra per unit: 32 (few prologues and power additions, the output's
+  // 16-spectra pieces whole), or fewer while that is less than two CTAs for
+  // every slot of the chip: 16 inputs x 128 channels x 100 spectra take 10.8 us
+  // at 2 against 18.9 us in fixed groups of 32 spectra a CTA.
   FeArgs b = a;
   const int slots = device_sm_count() * fe_min_blocks(LOGM);
   for (b.per_unit = 32; b.per_unit > 2; b.per_unit /= 2) {

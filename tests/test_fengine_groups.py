@@ -1,0 +1,51 @@
+"""How a channelise call is cut into groups of spectra changes nothing: one
+call over T spectra (32, 16, 8 ... spectra per FFT unit, as the size allows)
+equals the same spectra in short calls (two per unit), bit for bit, for gains
+on both sides of the bound where the equaliser needs no clamp."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("N,C,T,taps,low_gain", [
+    (192, 1024, 451, 4, False), (192, 64, 3700, 4, True), (192, 128, 1001, 3, False),
+    (100, 512, 200, 4, True), (191, 256, 300, 4, False), (192, 64, 3605, 6, False)])
+@pytest.mark.parametrize("layout", [0, 2])
+def test_one_call_is_its_slices(N, C, T, taps, low_gain, layout):
+    import torch
+    from paper_1904_07778_gb300.fengine import FEngine
+    M = 2 * C
+    g = torch.Generator(device="cuda").manual_seed(N + T)
+    adc = torch.randint(-127, 128, (N, (T + taps - 1) * M), generator=g, device="cuda", dtype=torch.int8)
+    gain = np.random.default_rng(T).integers(120, 6000, (C, N)).astype(np.uint32)
+    if low_gain:
+        gain[::3] = np.random.default_rng(C).integers(0, 140, gain[::3].shape)
+    gain[1, 0] = 0
+    with FEngine(N, C, taps) as f:
+        f.set_gains(gain)
+
+        def call(t0, n, stride):
+            out = torch.zeros((C, N, stride) if layout == 2 else (n, C, N), dtype=torch.uint8, device="cuda")
+            power = torch.zeros((C, N), dtype=torch.int64, device="cuda")
+            part = adc[:, t0 * M:(t0 + n + taps - 1) * M].contiguous()
+            f.channelise(part, n, out=out, layout=layout, out_stride=stride)
+            f.channelise(part, n, out=None, power=power)
+            f.sync()
+            return out, power
+
+        stride = (T + 15) // 16 * 16
+        whole, power = call(0, T, stride)
+        total = torch.zeros_like(power)
+        step = 24
+        for t0 in range(0, T, step):
+            n = min(step, T - t0)
+            part, p = call(t0, n, 24)
+            total += p
+            if layout == 2:
+                assert torch.equal(whole[:, :, t0:t0 + n], part[:, :, :n]), t0
+            else:
+                assert torch.equal(whole[t0:t0 + n], part), t0
+        assert torch.equal(power, total)
+        if layout == 2:
+            assert int(whole[:, :, T:].count_nonzero()) == 0   # nothing past the spectra
