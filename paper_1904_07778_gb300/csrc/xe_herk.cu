@@ -80,9 +80,14 @@ __device__ __forceinline__ int slot_block(const TaskGeom& g, int s) {
   return s == 0 ? g.cb0 : (s < g.nb ? g.cb1 : g.rb);
 }
 
-__device__ __forceinline__ void raise_timeout(int* status, volatile int* abort) {
+// Record a status bit, and for the host that there is one to read.
+__device__ __forceinline__ void raise_status(const HerkArgs& a, int bit) {
+  atomicOr(a.status, bit);
+  if (a.host_flag) *(volatile int*)a.host_flag = 1;
+}
+__device__ __forceinline__ void raise_timeout(const HerkArgs& a, volatile int* abort) {
   *abort = 1;
-  atomicOr(status, kStTimeout);
+  raise_status(a, kStTimeout);
 }
 
 __device__ __forceinline__ uint32_t swz_offset(int row, int chunk) {
@@ -259,14 +264,14 @@ __device__ __forceinline__ void tci8_keep(int c, int sw8, int lim, uint32_t (&ke
 // in slots 0..nb-1 (contiguous) and the A rows in slot a_slot.
 __device__ __forceinline__ void mma_loop(const TaskGeom& g, int nk, int nst, uint32_t ops_addr,
                                          uint32_t stage_bytes, uint32_t tmem, uint64_t* full,
-                                         uint64_t* empty, uint64_t* done, int* status,
+                                         uint64_t* empty, uint64_t* done, const HerkArgs& args,
                                          volatile int* abort) {
   const uint32_t idesc = umma_idesc(0, 128, 128 * g.nb);
   int s = 0;
   uint32_t ph = 0;
   for (int k = 0; k < nk; ++k) {
     if (!mbar_wait(&full[s], ph, abort)) {
-      raise_timeout(status, abort);
+      raise_timeout(args, abort);
       break;
     }
     tc_after_sync();
@@ -554,6 +559,8 @@ static_assert(regs_fit<false, false>() && regs_fit<true, false>() && regs_fit<fa
 #ifndef XE_MAX_SLOTS
 #define XE_MAX_SLOTS 16
 #endif
+// named barriers: 1 the drain warps, 2 .. the unpack groups, then the start
+constexpr int kStartBar = 2 + kGroups;
 constexpr int kMaxSlots = XE_MAX_SLOTS;  // ring slots at most (shared memory sets the count)
 static_assert(kEpiWarps % 4 == 0, "drain warps cover the four tensor-memory lane quarters");
 static_assert(kEpiWarps / 4 <= 2 && 16 * 4 * 128 == kHerkScratchInt2,
@@ -573,9 +580,17 @@ struct RingCtrl {
   alignas(16) int32_t usum[2][kMaxBlocks * 128];  // read by the drain in 16-byte loads
 };
 
-// Task j of this CTA: its explicit list, or round robin over the CTAs.
+// Task j of this CTA: its explicit list, or round robin over the CTAs.  The
+// tasks of a stacked array are one tile of channels each and are counted out
+// here (task_chans > 0): every role would otherwise read its next task from
+// memory, about 650 cycles at each task's start.
 __device__ __forceinline__ HerkTask my_task(const HerkArgs& a, int j) {
-  return a.cta_first ? a.tasks[a.cta_first[blockIdx.x] + j] : a.tasks[blockIdx.x + j * gridDim.x];
+  const int e = blockIdx.x + j * gridDim.x;
+  if (a.task_chans > 0) {
+    const int inst = a.insts ? e / a.tasks_per_inst : 0;
+    return {(e - inst * a.tasks_per_inst) * a.task_chans, 0, {0, -1}, inst};
+  }
+  return a.cta_first ? a.tasks[a.cta_first[blockIdx.x] + j] : a.tasks[e];
 }
 __device__ __forceinline__ int my_task_count(const HerkArgs& a) {
   if (a.cta_first) return a.cta_first[blockIdx.x + 1] - a.cta_first[blockIdx.x];
@@ -620,7 +635,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
   int ns = (int)(reinterpret_cast<uint8_t*>(&sm) - ring) / slot_bytes;
   if (ns > kMaxSlots) ns = kMaxSlots;
   if (ns < kGroups) {  // the host sizes shared memory for at least four slots
-    if (tid == 0) atomicOr(a.status, kStTimeout);
+    if (tid == 0) raise_status(a, kStTimeout);
     return;
   }
   volatile int* abort = &sm.abort;
@@ -628,28 +643,36 @@ __global__ void __launch_bounds__(kRingThreads, 1)
   // fault-injection tests shorten it), read from the parameter space at each wait
 #define budget ((!EIGHT && (a.in.fault >> 24)) ? (a.in.fault >> 24) : 31)
 
-  if (tid == 0) {
-    for (int s = 0; s < ns; ++s) {
-      mbar_init(&sm.full_t[s], 1);
-      mbar_init(&sm.full_o[s], kGroupWarps);
-      mbar_init(&sm.empty[s], 1);
+  // The loader sets up the barriers and does not wait for the other warps'
+  // part (row sums, tensor memory): its first loads are on their way while
+  // they prepare.
+  if (warp == kTmaWarp) {
+    if (lane == 0) {
+      for (int s = 0; s < ns; ++s) {
+        mbar_init(&sm.full_t[s], 1);
+        mbar_init(&sm.full_o[s], kGroupWarps);
+        mbar_init(&sm.empty[s], 1);
+      }
+      for (int b = 0; b < 2; ++b) {
+        mbar_init(&sm.tmem_full[b], 1);
+        mbar_init(&sm.tmem_empty[b], kEpiWarps);
+        mbar_init(&sm.usum_full[b], kUnpackWarps);
+        mbar_init(&sm.usum_empty[b], kEpiWarps);
+      }
+      mbar_init(&sm.done, 1);
+      sm.abort = 0;
+      fence_mbar_init();
     }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&sm.tmem_full[b], 1);
-      mbar_init(&sm.tmem_empty[b], kEpiWarps);
-      mbar_init(&sm.usum_full[b], kUnpackWarps);
-      mbar_init(&sm.usum_empty[b], kEpiWarps);
-    }
-    mbar_init(&sm.done, 1);
-    sm.abort = 0;
+    __syncwarp();
+    named_bar_arrive(kStartBar, kRingThreads);
+  } else {
+    for (int i = tid; i < 2 * kMaxBlocks * 128; i += blockDim.x) (&sm.usum[0][0])[i] = kUsumZero;
+    if (warp == 0) tmem_alloc(&sm.tmem_base, 512);
+    tc_before_sync();
+    named_bar_sync(kStartBar, kRingThreads);
+    tc_after_sync();
   }
-  for (int i = tid; i < 2 * kMaxBlocks * 128; i += blockDim.x) (&sm.usum[0][0])[i] = kUsumZero;
-  if (warp == 0) tmem_alloc(&sm.tmem_base, 512);
-  fence_mbar_init();
-  tc_before_sync();
-  __syncthreads();
-  tc_after_sync();
-  const uint32_t tmem = sm.tmem_base;
+  const uint32_t tmem = warp == kTmaWarp ? 0u : sm.tmem_base;
   const uint32_t ring_addr = smem_addr(ring);
   // Each role branch resizes its registers first: a setmaxnreg whose branches
   // joined again would leave the compiler the smaller budget for all roles.
@@ -682,7 +705,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
           stacked = in.rows_per_chan > 0;
         }
         if (m > 0 && !mbar_wait(&sm.empty[s], (uint32_t)((m - 1) & 1), abort, budget)) {
-          raise_timeout(a.status, abort);
+          raise_timeout(a, abort);
           break;
         }
         const int t = in.t0 + k * (kT << g.dbl);
@@ -730,7 +753,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
           const int k0 = EIGHT ? q * piece_stages<EIGHT>(g.dbl) : 0;
           const int k1 = EIGHT ? min(nk, k0 + piece_stages<EIGHT>(g.dbl)) : nk;
           if (v >= 2 && !mbar_wait(&sm.tmem_empty[b], (uint32_t)(((v >> 1) - 1) & 1), abort, budget)) {
-            raise_timeout(a.status, abort);
+            raise_timeout(a, abort);
             ok = false;
             break;
           }
@@ -741,7 +764,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
             constexpr bool dbl = decltype(DBL)::value;
             for (int k = k0; k < k1; ++k) {
               if (!mbar_wait(&sm.full_o[s], (uint32_t)(m & 1), abort, budget)) {
-                raise_timeout(a.status, abort);
+                raise_timeout(a, abort);
                 ok = false;
                 break;
               }
@@ -777,7 +800,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
       }
       umma_commit(&sm.done);
       int never = 0;
-      if (!mbar_wait(&sm.done, 0, &never, budget)) raise_timeout(a.status, abort);
+      if (!mbar_wait(&sm.done, 0, &never, budget)) raise_timeout(a, abort);
     }
     __syncwarp();
   } else if (warp < kUnpackWarps) {
@@ -832,7 +855,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
         const int k = S - S0;
         bool got = (m == 0 || mbar_wait(&sm.empty[s], (uint32_t)((m - 1) & 1), abort, budget)) &&
                    mbar_wait(&sm.full_t[s], (uint32_t)(m & 1), abort, budget);
-        if (!got) raise_timeout(a.status, abort);
+        if (!got) raise_timeout(a, abort);
         const uint32_t so = (uint32_t)(s * slot_bytes);
         const bool tail = (k + 1) * kTs > tn;
         // The operands of unit 0 overlap neither unit's packed bytes
@@ -947,7 +970,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
       }
       // publish this task's row sums once the buffer is free again
       const bool freed = j < 2 || mbar_wait(&sm.usum_empty[b], (uint32_t)(((j >> 1) - 1) & 1), abort, budget);
-      if (!freed) raise_timeout(a.status, abort);
+      if (!freed) raise_timeout(a, abort);
       if (!named_bar_and(2 + grp, kGroupThreads, freed)) break;
       if constexpr (TCI) {
         // the two lanes of a quad exchange planes, then each adds its own
@@ -968,7 +991,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.usum_full[b]);
     }
-    if (EIGHT && __any_sync(0xFFFFFFFFu, bad != 0) && lane == 0) atomicOr(a.status, kStRange);
+    if (EIGHT && __any_sync(0xFFFFFFFFu, bad != 0) && lane == 0) raise_status(a, kStRange);
   } else if (warp < kEpiWarp0) {
     regs_shrink<regs_other<LO_IS_REAL, EIGHT>()>();  // the two idle warps of the MMA / TMA warpgroup
   } else {
@@ -988,7 +1011,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
         const uint32_t par = (uint32_t)((v >> 1) & 1);
         const bool got = mbar_wait(&sm.tmem_full[b], par, abort, budget) &&
                          (EIGHT || mbar_wait(&sm.usum_full[b], par, abort, budget));
-        if (!got) raise_timeout(a.status, abort);
+        if (!got) raise_timeout(a, abort);
         if (!named_bar_and(1, kEpiWarps * 32, got)) {  // the drain warps leave together
           ok = false;
           break;
@@ -1027,7 +1050,7 @@ __global__ void __launch_bounds__(kLdgThreads, 1) herk4_ldg_kernel(const HerkArg
   extern __shared__ uint8_t dyn_raw[];
   __shared__ Ctrl sm;
   uint8_t* ops = align1024(dyn_raw);
-  const HerkTask task = args.tasks[blockIdx.x];
+  const HerkTask task = my_task(args, 0);  // one task a CTA
   const TaskGeom g = task_geom(task);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool stacked = a.rows_per_chan > 0;
@@ -1054,7 +1077,7 @@ __global__ void __launch_bounds__(kLdgThreads, 1) herk4_ldg_kernel(const HerkArg
   if (warp == 4) {
     if (lane == 0)
       mma_loop(g, nk, nst, smem_addr(ops), (uint32_t)stage_bytes, tmem, sm.full_o, sm.empty_o,
-               &sm.done, args.status, abort);
+               &sm.done, args, abort);
     __syncwarp();
   } else {
     const int chunk = tid & 7;
@@ -1086,7 +1109,7 @@ __global__ void __launch_bounds__(kLdgThreads, 1) herk4_ldg_kernel(const HerkArg
     uint32_t ph = 0;
     for (int k = 0; k < nk; ++k) {
       if (k >= nst && !mbar_wait(&sm.empty_o[s], ph ^ 1u, abort)) {
-        raise_timeout(args.status, abort);
+        raise_timeout(args, abort);
         break;
       }
       uint8_t* st = ops + s * stage_bytes;
@@ -1135,7 +1158,7 @@ __global__ void __launch_bounds__(kLdgThreads, 1) herk4_ldg_kernel(const HerkArg
     int never = 0;
     bool good = mbar_wait(&sm.done, 0, &never);
     good = __all_sync(0xFFFFFFFFu, good);
-    if (!good && lane == 0) raise_timeout(args.status, abort);
+    if (!good && lane == 0) raise_timeout(args, abort);
     tc_after_sync();
     if (good && !*abort)
       epilogue<false>(a, task, g, sm.usum, tmem, warp & 3, 0, 1, lane, true, true, nullptr);

@@ -71,7 +71,13 @@ struct HerkArgs {
   const HerkTask* tasks;
   const int* cta_first;      // if set, CTA b runs tasks [cta_first[b], cta_first[b + 1]);
                              // otherwise task j of CTA b is b + j * gridDim.x
+  // Stacked arrays, without a list (tasks unused): task e is the tile of
+  // channels task_chans (e mod tasks_per_inst) .. of instance
+  // e / tasks_per_inst (0 without insts).  0: the list.
+  int task_chans;
+  int tasks_per_inst;
   int* status;
+  int* host_flag;            // if set, mapped host memory that any status bit makes 1
   int lo_is_real;            // 4-bit: real part in the low nibble (whole launch)
   int bits;                  // 4, or 8 (byte rows: 2 per input, each one row of Y)
   // 8-bit: per-CTA partial sums of tasks longer than one accumulation,
