@@ -432,20 +432,21 @@ __global__ void pad_rows_kernel(const uint8_t* __restrict__ in, uint8_t* __restr
 // ---------------------------------------------------------------- normalise
 // rho = V / sqrt(V_ii V_jj) for a range of one channel's baselines.
 //
-// Bound: the FP64 pipe, which on this chip is 80 times narrower than FP32,
-// far ahead of the 32 bytes a baseline moves.  So the
-// square root and the two divisions of a baseline are not called: a block
-// keeps y_i = 1 / sqrt(V_ii) of its channel's inputs in shared memory (one
-// rsqrt per input, not per baseline), y_i y_j is the reciprocal of the
-// denominator to within a few ulp, and one FMA residual step each rounds the
-// square root and the quotients exactly as sqrt and / do (Markstein's
-// correction: s + (x - s^2) y / 2 and q + (a - q d) y with exact residuals;
-// compared with sqrt and / over 6e7 random operands without a difference).
-// That is 11 FP64 operations a baseline.  The baseline's inputs come from an
-// FP32 square root and integers.
-// The FP64 pipe runs 1.59 FMAs a cycle per SM here (measured), so 192 inputs x
-// 1024 channels need 0.42 ms of it; the call takes 0.471 ms, against 1.70 ms
-// with sqrt and two divisions a baseline.
+// Bound: the FP64 pipe, which on this chip is 80 times narrower than FP32
+// (1.59 FMAs a cycle per SM, measured), far ahead of the 32 bytes a baseline
+// moves.  So the square root and the two divisions of a baseline are not
+// called.  A block keeps 1 / sqrt(V_ii) and sqrt(V_ii) of its channel's inputs
+// in shared memory (one rsqrt per input, not per baseline) as float pairs;
+// their products, and those with V's parts, give the reciprocal of the
+// denominator, the denominator and the quotients to about 2^-46 in FP32 and
+// integer operations; and one FMA residual step each, exact to well below the
+// last bit, rounds the square root and the quotients as sqrt and / do
+// (Markstein's correction: s + (x - s^2) y / 2 and q + (a - q d) y; compared
+// with sqrt and / over 3e9 random operands without a difference).  That
+// leaves 7 FP64 operations a baseline, 0.27 ms of the pipe for 192 inputs x
+// 1024 channels: the call takes 345 us, 471 us with the estimates in FP64
+// too (11 operations), 1700 us with sqrt and two divisions.  The baseline's
+// inputs come from an FP32 square root and integers.
 constexpr int kNormThreads = 256;
 
 // (double)v without the FP64 pipe (the conversion instruction costs about
@@ -462,10 +463,32 @@ __device__ __forceinline__ double s64_to_double(long long v) {
   return __hiloint2double((int)hi, (int)(m << 21));
 }
 
+// The float pair a + b (|b| well below |a|; a normal, at least 2^-75 in
+// magnitude) as a double, in integers: the pair is renormalised (fast
+// two-sum), and its low part, in units of the high part's double ulp, is added
+// to the high part's widened bits.
+__device__ __forceinline__ double widen(float a, float b) {
+  const float h = a + b, e = b - (h - a);  // |e| <= half an ulp of h
+  const uint32_t u = __float_as_uint(h) & 0x7FFFFFFFu;
+  const float ulps = __uint_as_float((306u - (u >> 23)) << 23);  // 2^52 over h's power of two
+  int i = __float2int_rn(e * ulps);
+  if (h < 0.f) i = -i;
+  if ((u << 9) == 0 && i < 0) i *= 2;  // h a power of two: the ulp below it is half
+  const long long d = ((long long)u << 29) + (896ll << 52) + i;
+  return __longlong_as_double(d | ((long long)(__float_as_uint(h) & 0x80000000u) << 32));
+}
+
+// An input's factors: the power V_ii, and 1 / sqrt(V_ii) and sqrt(V_ii) as
+// float pairs.
+struct NormInput {
+  double p;
+  float yh, yl, rh, rl;
+};
+
 __global__ void __launch_bounds__(kNormThreads)
     normalise_kernel(const int64_t* __restrict__ acc, double* __restrict__ rho,
                      uint8_t* __restrict__ zero_flag, int nbl, int per_block, int vec_ok) {
-  extern __shared__ double norm_sm[];  // [2 i] = V_ii, [2 i + 1] = 1 / sqrt(V_ii)
+  extern __shared__ __align__(16) NormInput norm_sm[];
   const long long c = blockIdx.y;
   const int b0 = blockIdx.x * per_block, b1 = min(nbl, b0 + per_block);
   const int64_t* v = acc + c * nbl * 2;
@@ -477,9 +500,14 @@ __global__ void __launch_bounds__(kNormThreads)
   };
   const int last = input_of(b1 - 1);  // no baseline of the range has a larger input
   for (int i = threadIdx.x; i <= last; i += kNormThreads) {
-    const double p = (double)v[i * (i + 3)];
-    norm_sm[2 * i] = p;
-    norm_sm[2 * i + 1] = rsqrt(fabs(p));
+    NormInput n;
+    n.p = (double)v[i * (i + 3)];
+    const double y = rsqrt(fabs(n.p)), r = fabs(n.p) * y;
+    n.yh = (float)y;
+    n.yl = (float)(y - (double)n.yh);
+    n.rh = (float)r;
+    n.rl = (float)(r - (double)n.rh);
+    norm_sm[i] = n;
   }
   __syncthreads();
   for (int b = b0 + (int)threadIdx.x; b < b1; b += kNormThreads) {
@@ -492,21 +520,35 @@ __global__ void __launch_bounds__(kNormThreads)
       vr = v[2 * b];
       vi = v[2 * b + 1];
     }
-    const double2 pi = reinterpret_cast<const double2*>(norm_sm)[i];
-    const double2 pj = reinterpret_cast<const double2*>(norm_sm)[j];
-    const double den2 = pi.x * pj.x;
+    const NormInput ni = norm_sm[i], nj = norm_sm[j];
+    const double den2 = ni.p * nj.p;
     double re = 0.0, im = 0.0;
     const int top = __double2hiint(den2);  // |den2| is 0 or at least 1: its sign and zero from the high word
     if (top > 0) {
-      const double y = pi.y * pj.y;
-      const double s = den2 * y;
+      // 1 / sqrt(den2) and sqrt(den2) to about 2^-46, as float pairs
+      const float yh = ni.yh * nj.yh;
+      const float yl = fmaf(ni.yl, nj.yh, fmaf(ni.yh, nj.yl, fmaf(ni.yh, nj.yh, -yh)));
+      const float sh = ni.rh * nj.rh;
+      const float sl = fmaf(ni.rl, nj.rh, fmaf(ni.rh, nj.rl, fmaf(ni.rh, nj.rh, -sh)));
+      const double y = widen(yh, yl), s = widen(sh, sl);
       // y / 2: one off the exponent (y is a normal number: powers are >= 1)
       const double h = __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y));
       const double den = fma(fma(-s, s, den2), h, s);
-      const double xr = s64_to_double(vr), xi = s64_to_double(vi);
-      const double qr = xr * y, qi = xi * y;
-      re = fma(fma(-qr, den, xr), y, qr);
-      im = fma(fma(-qi, den, xi), y, qi);
+      auto divide = [&](long long w) {
+        const int x = (int)w;
+        double q;
+        if (w == (long long)x && abs(x) < (1 << 30)) {
+          if (x == 0) return 0.0;
+          const float xh = (float)x, xl = (float)(x - __float2int_rn(xh));
+          const float qh = xh * yh;
+          q = widen(qh, fmaf(xl, yh, fmaf(xh, yl, fmaf(xh, yh, -qh))));
+        } else {
+          q = (double)w * y;
+        }
+        return fma(fma(-q, den, s64_to_double(w)), y, q);
+      };
+      re = divide(vr);
+      im = divide(vi);
     } else if ((top << 1) != 0) {
       re = im = sqrt(den2);  // not a power: NaN
     }
@@ -643,7 +685,7 @@ cudaError_t normalise_launch(const int64_t* acc, double* rho, uint8_t* zero_flag
   const int want = std::max(1, device_sm_count() * 32 / n_chans);
   const int per = std::max(kNormThreads, (nbl + want - 1) / want);
   const int vec_ok = reinterpret_cast<uintptr_t>(acc) % 16 == 0 && reinterpret_cast<uintptr_t>(rho) % 16 == 0;
-  const size_t smem = (size_t)n_inputs * 2 * sizeof(double);
+  const size_t smem = (size_t)n_inputs * sizeof(NormInput);
   for (int c0 = 0; c0 < n_chans; c0 += 65535) {  // grid.y
     const int nc = std::min(65535, n_chans - c0);
     const long long e0 = (long long)c0 * nbl;
