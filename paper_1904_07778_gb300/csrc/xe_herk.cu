@@ -80,6 +80,35 @@ __device__ __forceinline__ int slot_block(const TaskGeom& g, int s) {
   return s == 0 ? g.cb0 : (s < g.nb ? g.cb1 : g.rb);
 }
 
+// A task of a pair of CTAs (HerkArgs::pair): the 256 x 256 block of super row
+// t.rb (row blocks 2 t.rb, 2 t.rb + 1) and super column t.cb[0], t.cb[0] <=
+// t.rb.  CTA `rank` has the A rows of block 2 t.rb + rank and the B rows of
+// block 2 t.cb[0] + rank; the tensor core reads both CTAs' B.  On the diagonal
+// A = B, and CTA 0 leaves its second column block (the transpose of one of
+// CTA 1's) unread.
+__device__ __forceinline__ TaskGeom pair_geom(const HerkTask& t, int rank) {
+  TaskGeom g;
+  g.rb = 2 * t.rb + rank;
+  g.cb0 = 2 * t.cb[0];
+  g.cb1 = g.cb0 + 1;
+  g.dbl = t.rb == t.cb[0] ? 1 : 0;
+  g.nb = g.dbl && rank == 0 ? 1 : 2;
+  g.nblk = g.dbl ? 1 : 2;
+  g.a_slot = g.dbl ? 0 : 1;
+  g.ncols = 256u;
+  return g;
+}
+template <bool PAIR>
+__device__ __forceinline__ TaskGeom geom(const HerkTask& t, int rank) {
+  return PAIR ? pair_geom(t, rank) : task_geom(t);
+}
+// Row block of unit u of a stage (double stages: the same block twice).
+template <bool PAIR>
+__device__ __forceinline__ int unit_block(const TaskGeom& g, int u, int rank) {
+  if (PAIR) return g.dbl || u == 1 ? g.rb : g.cb0 + rank;
+  return slot_block(g, g.dbl ? 0 : u);
+}
+
 // Record a status bit, and for the host that there is one to read.
 __device__ __forceinline__ void raise_status(const HerkArgs& a, int bit) {
   atomicOr(a.status, bit);
@@ -336,7 +365,7 @@ __device__ __forceinline__ void epilogue(const HerkInst& a, const HerkTask& task
   for (int h = 0; h < 2; ++h) {  // the quarter's 16-row halves
     const int gr = 2 * quad + h;            // the half's group of 8 samples
     const int m = 8 * gr + (lane >> 3) + (lane & 4);  // the thread's sample
-    int ch = task.chan0, i = task.rb * 64 + m;
+    int ch = task.chan0, i = g.rb * 64 + m;
     if (half) {
       ch += m >> (31 - __clz(half));
       i = m & (half - 1);
@@ -433,8 +462,8 @@ __device__ __forceinline__ void epilogue(const HerkInst& a, const HerkTask& task
 #pragma unroll 1
       for (int s = 0; s < g.nb; ++s) {
         const int cblk = slot_block(g, s);
-        if (cblk <= task.rb) {  // the diagonal block up to the rows' group, or a lower block
-          row_walk(8 * s, cblk == task.rb ? gr + 1 : 8, 64 * cblk);
+        if (cblk <= g.rb) {  // the diagonal block up to the rows' group, or a lower block
+          row_walk(8 * s, cblk == g.rb ? gr + 1 : 8, 64 * cblk);
         } else {  // baselines (j, i), j > i: the conjugate
           const int jb = 64 * cblk + q0;
           walk(8 * s, part, 8, [&](int k, int re0, int im0, int re1, int im1) {
@@ -584,17 +613,21 @@ struct RingCtrl {
 // tasks of a stacked array are one tile of channels each and are counted out
 // here (task_chans > 0): every role would otherwise read its next task from
 // memory, about 650 cycles at each task's start.
+template <bool PAIR = false>
 __device__ __forceinline__ HerkTask my_task(const HerkArgs& a, int j) {
-  const int e = blockIdx.x + j * gridDim.x;
-  if (a.task_chans > 0) {
+  const int c = PAIR ? blockIdx.x >> 1 : blockIdx.x;  // a pair of CTAs walks its tasks together
+  const int e = c + j * (PAIR ? gridDim.x >> 1 : gridDim.x);
+  if (!PAIR && a.task_chans > 0) {
     const int inst = a.insts ? e / a.tasks_per_inst : 0;
     return {(e - inst * a.tasks_per_inst) * a.task_chans, 0, {0, -1}, inst};
   }
-  return a.cta_first ? a.tasks[a.cta_first[blockIdx.x] + j] : a.tasks[e];
+  return a.cta_first ? a.tasks[a.cta_first[c] + j] : a.tasks[e];
 }
+template <bool PAIR>
 __device__ __forceinline__ int my_task_count(const HerkArgs& a) {
-  if (a.cta_first) return a.cta_first[blockIdx.x + 1] - a.cta_first[blockIdx.x];
-  return (a.n_tasks - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+  const int c = PAIR ? blockIdx.x >> 1 : blockIdx.x, n = PAIR ? gridDim.x >> 1 : gridDim.x;
+  if (a.cta_first) return a.cta_first[c + 1] - a.cta_first[c];
+  return (a.n_tasks - c + n - 1) / n;
 }
 __device__ __forceinline__ HerkInst task_inst(const HerkArgs& a, const HerkTask& t) {
   return a.insts ? a.insts[t.inst] : a.in;
@@ -618,9 +651,19 @@ __device__ __forceinline__ int pieces_of(int nk, int dbl) {
 
 // TCI: the tensor maps describe payload-order blocks ({byte row, channel,
 // time}) and the unpack transposes.  EIGHT: 8-bit samples as FP16 operands.
-template <bool LO_IS_REAL, bool EIGHT, bool TCI>
+// PAIR (8-bit): clusters of two CTAs share tasks of 256 x 256 (pair_geom).
+// What bounds a stage is shared memory (the MMAs run at about 200 cycles each
+// against 128 alone): per CTA the TMA's 16 KB in, read back by the unpack, 32
+// KB of operands written, and the MMA's reads, 16 KB of A and 32 KB of B for
+// two 128 x 128 blocks.  In a pair each CTA feeds half of B to both (16 KB),
+// and large arrays need no 128 x 128 tasks, which load two blocks for one: 96
+// KB a stage for two blocks (64 KB on the diagonal) against 112 KB for two and
+// 96 KB for one.  Measured (push and dump, T = 4096): 512 inputs x 304 channels
+// 1.72 -> 1.13 ms, 384 x 304 0.955 -> 0.676, 256 x 608 0.809 -> 0.667.
+template <bool LO_IS_REAL, bool EIGHT, bool TCI, bool PAIR>
 __global__ void __launch_bounds__(kRingThreads, 1)
     herk4_ring_kernel(const __grid_constant__ CUtensorMap tmap, const HerkArgs a) {
+  static_assert(!PAIR || EIGHT, "pairs exchange no row sums");
   constexpr int kT = stage_t<EIGHT>();             // spectra per stage
   constexpr int kPkRowBytes = kT;                  // packed bytes of a byte row in a stage
   extern __shared__ uint8_t dyn_raw[];
@@ -630,7 +673,8 @@ __global__ void __launch_bounds__(kRingThreads, 1)
       dyn_raw + ((a.smem_bytes - (int)sizeof(RingCtrl)) & ~15));
   uint8_t* ring = align1024(dyn_raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n_my = my_task_count(a);  // tasks of this CTA; stage counts vary per array
+  const int rank = PAIR ? (int)cluster_rank() : 0;
+  const int n_my = my_task_count<PAIR>(a);  // tasks of this CTA; stage counts vary per array
   constexpr int slot_bytes = kSlotBytes;
   int ns = (int)(reinterpret_cast<uint8_t*>(&sm) - ring) / slot_bytes;
   if (ns > kMaxSlots) ns = kMaxSlots;
@@ -650,12 +694,12 @@ __global__ void __launch_bounds__(kRingThreads, 1)
     if (lane == 0) {
       for (int s = 0; s < ns; ++s) {
         mbar_init(&sm.full_t[s], 1);
-        mbar_init(&sm.full_o[s], kGroupWarps);
+        mbar_init(&sm.full_o[s], (PAIR ? 2 : 1) * kGroupWarps);
         mbar_init(&sm.empty[s], 1);
       }
       for (int b = 0; b < 2; ++b) {
         mbar_init(&sm.tmem_full[b], 1);
-        mbar_init(&sm.tmem_empty[b], kEpiWarps);
+        mbar_init(&sm.tmem_empty[b], (PAIR ? 2 : 1) * kEpiWarps);
         mbar_init(&sm.usum_full[b], kUnpackWarps);
         mbar_init(&sm.usum_empty[b], kEpiWarps);
       }
@@ -664,12 +708,23 @@ __global__ void __launch_bounds__(kRingThreads, 1)
       fence_mbar_init();
     }
     __syncwarp();
-    named_bar_arrive(kStartBar, kRingThreads);
+    if (!PAIR) named_bar_arrive(kStartBar, kRingThreads);
   } else {
     for (int i = tid; i < 2 * kMaxBlocks * 128; i += blockDim.x) (&sm.usum[0][0])[i] = kUsumZero;
-    if (warp == 0) tmem_alloc(&sm.tmem_base, 512);
+    if (warp == 0) {
+      if (PAIR)
+        tmem_alloc_pair(&sm.tmem_base, 512);
+      else
+        tmem_alloc(&sm.tmem_base, 512);
+    }
     tc_before_sync();
-    named_bar_sync(kStartBar, kRingThreads);
+    if (!PAIR) named_bar_sync(kStartBar, kRingThreads);
+    tc_after_sync();
+  }
+  if (PAIR) {  // (the other CTA's barriers are set up too before anything arrives on them)
+    __syncwarp();
+    __syncthreads();
+    cluster_sync();
     tc_after_sync();
   }
   const uint32_t tmem = warp == kTmaWarp ? 0u : sm.tmem_base;
@@ -685,8 +740,8 @@ __global__ void __launch_bounds__(kRingThreads, 1)
       // for it run out and the CTA unwinds with a timeout status
       const int skip = (blockIdx.x == 0 && (a.in.fault & 0xFFFFFF) > 0) ? (a.in.fault & 0xFFFFFF) - 1 : -1;
       int s = 0, m = 0, j = 0, k = 0, issued = 0;
-      HerkTask task = my_task(a, 0);
-      TaskGeom g = task_geom(task);
+      HerkTask task = my_task<PAIR>(a, 0);
+      TaskGeom g = geom<PAIR>(task, rank);
       HerkInst in = task_inst(a, task);
       const CUtensorMap* tm = a.tmaps ? &a.tmaps[task.inst] : &tmap;
       if (a.tmaps) tensormap_acquire(tm);
@@ -696,8 +751,8 @@ __global__ void __launch_bounds__(kRingThreads, 1)
         if (k == nk) {  // next task
           if (++j == n_my) break;
           k = 0;
-          task = my_task(a, j);
-          g = task_geom(task);
+          task = my_task<PAIR>(a, j);
+          g = geom<PAIR>(task, rank);
           in = task_inst(a, task);
           tm = a.tmaps ? &a.tmaps[task.inst] : &tmap;
           if (a.tmaps) tensormap_acquire(tm);
@@ -716,7 +771,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
             const uint32_t dst = dst0 + (uint32_t)(u * kRPkBlock);
             // unit u: block u, or the block's second time range
             // (byte rows of a 128-row block: 64 at 4 bits, 128 at 8 bits)
-            const int row0 = stacked ? 0 : (kRPkBlock / kPkRowBytes) * slot_block(g, g.dbl ? 0 : u);
+            const int row0 = stacked ? 0 : (kRPkBlock / kPkRowBytes) * unit_block<PAIR>(g, u, rank);
             const int tu = t + (g.dbl ? u * kT : 0);
             if (TCI)
               tma_load_3d(dst, tm, row0, task.chan0, tu, &sm.full_t[s]);
@@ -739,15 +794,15 @@ __global__ void __launch_bounds__(kRingThreads, 1)
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------------ MMA issuer
     regs_shrink<regs_other<LO_IS_REAL, EIGHT>()>();
-    if (lane == 0) {
+    if (lane == 0 && rank == 0) {  // (a pair's MMAs are all issued by CTA 0)
       int s = 0, m = 0, v = 0;  // v: accumulations so far (tensor-memory buffer v & 1)
       bool ok = true;
       for (int j = 0; j < n_my && ok; ++j) {
-        const HerkTask task = my_task(a, j);
-        const TaskGeom g = task_geom(task);
+        const HerkTask task = my_task<PAIR>(a, j);
+        const TaskGeom g = geom<PAIR>(task, rank);
         const int nk = stages_of<EIGHT>(task_inst(a, task), g.dbl);
         const int np = pieces_of<EIGHT>(nk, g.dbl);
-        const uint32_t idesc = umma_idesc(0, 128, 128 * g.nb);
+        const uint32_t idesc = PAIR ? umma_idesc(0, 256, 256) : umma_idesc(0, 128, 128 * g.nb);
         for (int q = 0; q < np && ok; ++q, ++v) {
           const int b = v & 1;
           const int k0 = EIGHT ? q * piece_stages<EIGHT>(g.dbl) : 0;
@@ -779,12 +834,17 @@ __global__ void __launch_bounds__(kRingThreads, 1)
                 const uint64_t da = dbl ? bdesc + (uint64_t)((kk >> 2) * (kROpBlock >> 4) + 2 * (kk & 3))
                                         : adesc + 2 * kk;
                 const uint64_t db = dbl ? da : bdesc + 2 * kk;
-                if (EIGHT)
+                if (PAIR)
+                  umma_f16_pair(d, da, db, idesc, (k != k0 || kk != 0));
+                else if (EIGHT)
                   umma_f16(d, da, db, idesc, (k != k0 || kk != 0));
                 else
                   umma_f8(d, da, db, idesc, (k != k0 || kk != 0));
               }
-              umma_commit(&sm.empty[s]);
+              if (PAIR)
+                umma_commit_pair(&sm.empty[s]);
+              else
+                umma_commit(&sm.empty[s]);
               if (++s == ns) {
                 s = 0;
                 ++m;
@@ -795,10 +855,18 @@ __global__ void __launch_bounds__(kRingThreads, 1)
             issue(std::true_type{});
           else
             issue(std::false_type{});
-          if (ok) umma_commit(&sm.tmem_full[b]);
+          if (ok) {
+            if (PAIR)
+              umma_commit_pair(&sm.tmem_full[b]);
+            else
+              umma_commit(&sm.tmem_full[b]);
+          }
         }
       }
-      umma_commit(&sm.done);
+      if (PAIR)
+        umma_commit_pair(&sm.done);
+      else
+        umma_commit(&sm.done);
       int never = 0;
       if (!mbar_wait(&sm.done, 0, &never, budget)) raise_timeout(a, abort);
     }
@@ -841,8 +909,8 @@ __global__ void __launch_bounds__(kRingThreads, 1)
     int S0 = 0;  // first stage of task j
     for (int j = 0; j < n_my && ok; ++j) {
       const int b = j & 1;
-      const HerkTask task = my_task(a, j);
-      const TaskGeom g = task_geom(task);
+      const HerkTask task = my_task<PAIR>(a, j);
+      const TaskGeom g = geom<PAIR>(task, rank);
       const int tn = task_inst(a, task).tn;
       const int kTs = kT << g.dbl;  // spectra per stage of this task
       const int S1 = S0 + (tn + kTs - 1) / kTs;
@@ -951,7 +1019,12 @@ __global__ void __launch_bounds__(kRingThreads, 1)
         store(std::integral_constant<int, 1>{});
         fence_smem_to_async();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.full_o[s]);
+        if (lane == 0) {
+          if (PAIR)
+            mbar_arrive_cluster(&sm.full_o[s], 0);
+          else
+            mbar_arrive(&sm.full_o[s]);
+        }
         s += kGroups;
         if (s >= ns) {
           s -= ns;
@@ -1002,9 +1075,9 @@ __global__ void __launch_bounds__(kRingThreads, 1)
     int v = 0;
     bool ok = true;
     for (int j = 0; j < n_my && ok; ++j) {
-      const HerkTask task = my_task(a, j);
+      const HerkTask task = my_task<PAIR>(a, j);
       const HerkInst in = task_inst(a, task);
-      const TaskGeom g = task_geom(task);
+      const TaskGeom g = geom<PAIR>(task, rank);
       const int np = pieces_of<EIGHT>(stages_of<EIGHT>(in, g.dbl), g.dbl);
       for (int q = 0; q < np; ++q, ++v) {
         const int b = v & 1;
@@ -1021,7 +1094,12 @@ __global__ void __launch_bounds__(kRingThreads, 1)
                         kEpiWarps / 4, lane, q == 0, q == np - 1, scr);
         tc_before_sync();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.tmem_empty[b]);
+        if (lane == 0) {
+          if (PAIR)
+            mbar_arrive_cluster(&sm.tmem_empty[b], 0);
+          else
+            mbar_arrive(&sm.tmem_empty[b]);
+        }
         if (!EIGHT) {
           // every drain warp has read the sums: clear them for task j + 2
           named_bar_sync(1, kEpiWarps * 32);
@@ -1036,7 +1114,13 @@ __global__ void __launch_bounds__(kRingThreads, 1)
 #undef budget
   tc_before_sync();
   __syncthreads();
-  if (warp == 0) tmem_free(tmem, 512);
+  if (PAIR) cluster_sync();  // neither CTA's shared or tensor memory is in use by the other's work
+  if (warp == 0) {
+    if (PAIR)
+      tmem_free_pair(tmem, 512);
+    else
+      tmem_free(tmem, 512);
+  }
 }
 
 // -------------------------------------------------------------- LDG kernel
@@ -1185,27 +1269,44 @@ cudaError_t set_smem(K kernel, int bytes) {
 int ring_smem() {
   static int m = -1;
   if (m < 0)
-    m = std::min(std::min(max_dyn_smem((const void*)herk4_ring_kernel<false, false, false>),
-                          max_dyn_smem((const void*)herk4_ring_kernel<true, false, false>)),
-                 max_dyn_smem((const void*)herk4_ring_kernel<false, true, false>));
-    m = std::min(m, std::min(std::min(max_dyn_smem((const void*)herk4_ring_kernel<false, false, true>),
-                                      max_dyn_smem((const void*)herk4_ring_kernel<true, false, true>)),
-                             max_dyn_smem((const void*)herk4_ring_kernel<false, true, true>)));
+    m = std::min(std::min(max_dyn_smem((const void*)herk4_ring_kernel<false, false, false, false>),
+                          max_dyn_smem((const void*)herk4_ring_kernel<true, false, false, false>)),
+                 max_dyn_smem((const void*)herk4_ring_kernel<false, true, false, false>));
+    m = std::min(m, std::min(std::min(max_dyn_smem((const void*)herk4_ring_kernel<false, false, true, false>),
+                                      max_dyn_smem((const void*)herk4_ring_kernel<true, false, true, false>)),
+                             max_dyn_smem((const void*)herk4_ring_kernel<false, true, true, false>)));
+    m = std::min(m, std::min(max_dyn_smem((const void*)herk4_ring_kernel<false, true, false, true>),
+                             max_dyn_smem((const void*)herk4_ring_kernel<false, true, true, true>)));
   return m;
 }
 
-template <bool LO, bool EIGHT, bool TCI>
+template <bool LO, bool EIGHT, bool TCI, bool PAIR = false>
 cudaError_t ring_launch(const HerkArgs& a, const CUtensorMap* tmap, int grid, cudaStream_t s) {
   // the attribute persists: set it once, so that launches captured into a
   // CUDA graph are plain stream work
   static int set_bytes = -1;
   if (set_bytes != a.smem_bytes) {
-    cudaError_t e = set_smem(herk4_ring_kernel<LO, EIGHT, TCI>, a.smem_bytes);
+    cudaError_t e = set_smem(herk4_ring_kernel<LO, EIGHT, TCI, PAIR>, a.smem_bytes);
     if (e != cudaSuccess) return e;
     set_bytes = a.smem_bytes;
   }
-  herk4_ring_kernel<LO, EIGHT, TCI><<<grid, kRingThreads, a.smem_bytes, s>>>(*tmap, a);
-  return cudaGetLastError();
+  if constexpr (PAIR) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kRingThreads);
+    cfg.dynamicSmemBytes = a.smem_bytes;
+    cfg.stream = s;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 2;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, herk4_ring_kernel<LO, EIGHT, TCI, PAIR>, *tmap, a);
+  } else {
+    herk4_ring_kernel<LO, EIGHT, TCI, PAIR><<<grid, kRingThreads, a.smem_bytes, s>>>(*tmap, a);
+    return cudaGetLastError();
+  }
 }
 
 }  // namespace
@@ -1242,14 +1343,20 @@ cudaError_t herk4_launch(const HerkArgs& args, const CUtensorMap* tmap, int n_ta
     int grid;
     if (a.cta_first) {
       grid = a.grid;
+    } else if (a.pair) {  // two CTAs a task
+      grid = 2 * std::min(n_tasks, device_sm_count() / 2);
     } else {
       grid = std::min(n_tasks, device_sm_count());
       if (a.grid > 0) grid = std::min(grid, a.grid);
     }
     if (grid < 1) return cudaSuccess;
+    if (a.pair && (a.bits != 8 || grid % 2 != 0)) return cudaErrorInvalidValue;
     if (a.bits == 8 && (!a.scratch || grid > a.scratch_ctas)) return cudaErrorInvalidValue;
     static const CUtensorMap unused{};  // batched launches read their maps from a.tmaps
     const CUtensorMap* m = tmap ? tmap : &unused;
+    if (a.pair)
+      return tci ? ring_launch<false, true, true, true>(a, m, grid, s)
+                 : ring_launch<false, true, false, true>(a, m, grid, s);
     if (tci) {
       if (a.bits == 8) return ring_launch<false, true, true>(a, m, grid, s);
       return a.lo_is_real ? ring_launch<true, false, true>(a, m, grid, s)

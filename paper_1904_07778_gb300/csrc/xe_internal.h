@@ -76,6 +76,9 @@ struct HerkArgs {
   // e / tasks_per_inst (0 without insts).  0: the list.
   int task_chans;
   int tasks_per_inst;
+  // 8-bit: tasks are 256 x 256 blocks of clusters of two CTAs (plan_pair_tasks);
+  // cta_first and tasks are then per cluster, grid counts CTAs.
+  int pair;
   int* status;
   int* host_flag;            // if set, mapped host memory that any status bit makes 1
   int lo_is_real;            // 4-bit: real part in the low nibble (whole launch)
@@ -188,6 +191,11 @@ cudaError_t turn_rows_chans(const uint8_t* in, uint8_t* out, int layout, int bit
 // HerkTask): rows_per_chan is set for stacked arrays.  With singles, every
 // task has one column block (128 x 128).
 std::vector<HerkTask> plan_tasks(int n_inputs, int n_chans, int* rows_per_chan, bool singles = false);
+
+// The same in 256 x 256 tasks for pairs of CTAs: {channel, super row, {super
+// column, -1}}.  pair_tasks_pay: whether an array is better multiplied so.
+std::vector<HerkTask> plan_pair_tasks(int n_inputs, int n_chans);
+bool pair_tasks_pay(int bits, int n_inputs);
 
 // Snapshot the device status word into host_slot (pinned host memory, written
 // by the device through its mapping; read it once the stream has passed this

@@ -114,6 +114,26 @@ std::vector<HerkTask> plan_tasks(int n, int c, int* rows_per_chan, bool singles)
   return t;
 }
 
+std::vector<HerkTask> plan_pair_tasks(int n, int c) {
+  std::vector<HerkTask> t;
+  const int nsr = ((2 * n + 127) / 128 + 1) / 2;  // super rows of two 128-row blocks
+  for (int diag = 0; diag < 2; ++diag)  // the longer tasks first
+    for (int ch = 0; ch < c; ++ch)
+      for (int r = 0; r < nsr; ++r)
+        for (int k = diag ? r : 0; k < (diag ? r + 1 : r); ++k) t.push_back({ch, r, {k, -1}, 0});
+  return t;
+}
+
+// By the shared-memory traffic of a stage (the ring kernel's bound), per
+// channel: pairs move 2 x 96 KB per off-diagonal 256 x 256 task and 2 x 64 KB
+// per diagonal one (an odd count of row blocks leaves half of the last super
+// row empty); single CTAs 112 KB per 128 x 256 task and 96 KB per 128 x 128
+// one.  With three row blocks (129 .. 192 inputs) single CTAs move 336 KB, pairs
+// 448; from four on pairs move less.  Measured at 64 channels, push and dump:
+// 200 inputs (x 2048 spectra) 87 -> 78 us, 256 (128 channels, 4096) 217 -> 179,
+// 320 (1024) 68 -> 64, 448 (4096) 302 -> 272, 512 (4096) 391 -> 274.
+bool pair_tasks_pay(int bits, int n_inputs) { return bits == 8 && n_inputs > 192; }
+
 }  // namespace xe
 
 struct corr_ctx {
@@ -165,6 +185,11 @@ struct corr_ctx {
   long long turned_stride = 0;  // bytes per (channel, input) row of `turned`
   HerkTask* tasks = nullptr;
   int n_tasks = 0;
+  // pairs of CTAs (pair_tasks_pay): `tasks` are theirs, and a pipelined push,
+  // whose turn may sit on one SM of a pair, takes the single CTAs' list
+  bool pair = false;
+  HerkTask* single_tasks = nullptr;
+  int n_single_tasks = 0;
   int2* scratch = nullptr;  // 8-bit: per-CTA partial sums of the cross-multiply
   int scratch_ctas = 0;
   // host-side caches of the push path: two block addresses known to be device
@@ -334,6 +359,7 @@ void free_ctx(corr_ctx* x) {
   }
   cudaFree(x->turned);
   cudaFree(x->tasks);
+  cudaFree(x->single_tasks);
   cudaFree(x->scratch);
   cudaFree(x->d_status);
   cudaFree(x->rho_tmp);
@@ -502,6 +528,13 @@ int corr_create(int n_inputs, int n_chans, int n_time, int bits, int layout, uns
     }
     if (st != CORR_OK) break;
     std::vector<HerkTask> tasks = plan_tasks(n_inputs, n_chans, &x->rows_per_chan);
+    x->pair = pair_tasks_pay(bits, n_inputs);
+    if (x->pair && turn_can_persist(layout, bits)) {
+      x->n_single_tasks = (int)tasks.size();
+      if (cudaMalloc(&x->single_tasks, tasks.size() * sizeof(HerkTask)) != cudaSuccess) { st = CORR_ENOMEM; break; }
+      if (cudaMemcpy(x->single_tasks, tasks.data(), tasks.size() * sizeof(HerkTask), cudaMemcpyHostToDevice) != cudaSuccess) { st = CORR_ECUDA; break; }
+    }
+    if (x->pair) tasks = plan_pair_tasks(n_inputs, n_chans);
     x->n_tasks = (int)tasks.size();
     x->host_tasks = tasks;
     if (bits == 8 && herk_scratch_alloc(&x->scratch, &x->scratch_ctas) != cudaSuccess) { st = CORR_ENOMEM; break; }
@@ -606,7 +639,10 @@ int corr_push(corr_ctx* x, const void* block, size_t nbytes, uint64_t seq) {
   a.in.x = src;
   a.in.fault = x->fault;
   a.in.acc = x->acc;
-  a.tasks = x->tasks;
+  const bool pair = x->pair && !pipe;
+  const int n_tasks = x->pair && pipe ? x->n_single_tasks : x->n_tasks;
+  a.tasks = x->pair && pipe ? x->single_tasks : x->tasks;
+  a.pair = pair ? 1 : 0;
   if (x->rows_per_chan > 0) {
     a.task_chans = 128 / x->rows_per_chan;
     a.tasks_per_inst = x->n_tasks;
@@ -620,7 +656,7 @@ int corr_push(corr_ctx* x, const void* block, size_t nbytes, uint64_t seq) {
   a.in.rows_per_chan = x->rows_per_chan;
   a.lo_is_real = (x->flags & CORR_F_LO_IS_REAL) ? 1 : 0;
   a.smem_bytes = x->smem_bytes;
-  a.n_tasks = x->n_tasks;
+  a.n_tasks = n_tasks;
   a.bits = x->bits;
   a.scratch = x->scratch;
   a.scratch_ctas = x->scratch_ctas;
@@ -652,7 +688,7 @@ int corr_push(corr_ctx* x, const void* block, size_t nbytes, uint64_t seq) {
     a.in.accumulate = x->acc_live ? 1 : 0;
     a.in.vec_ok = aligned ? 1 : 0;
     cudaEvent_t th = phase_begin(x, hs);
-    cudaError_t e = herk4_launch(a, tmap, x->n_tasks, hs, tci);
+    cudaError_t e = herk4_launch(a, tmap, n_tasks, hs, tci);
     if (e != cudaSuccess) return cuda_fail(e);
     phase_end(x, kHerk, th, hs);
     ++x->stats.herk_launches;
@@ -792,6 +828,7 @@ int corr_push_many(corr_ctx* x, const void* const* blocks, int n_blocks, size_t 
   a.insts = tb->d_insts;
   a.tmaps = tb->d_maps;
   a.tasks = x->many_tasks;
+  a.pair = x->pair ? 1 : 0;
   if (x->rows_per_chan > 0) {
     a.task_chans = 128 / x->rows_per_chan;
     a.tasks_per_inst = x->n_tasks;

@@ -88,6 +88,7 @@ struct Req {
   size_t block_bytes = 0, acc_bytes = 0, turn_bytes = 0;
   bool has_turn = false;
   bool tci = false;  // blocks read in payload order (no corner turn)
+  bool pair = false;  // tasks of pairs of CTAs
   long long stride = 0;
   // arena offsets of the pieces (valid while admitted)
   size_t off_acc = 0, off_in[2] = {0, 0}, off_turn = 0;
@@ -198,6 +199,8 @@ void admit(corr_svc* s) {
     q.slot = s->free_slots.back();
     s->free_slots.pop_back();
     q.tasks = plan_tasks(q.r.n_inputs, q.r.n_chans, &q.rpc);
+    q.pair = pair_tasks_pay(q.r.bits, q.r.n_inputs);
+    if (q.pair) q.tasks = plan_pair_tasks(q.r.n_inputs, q.r.n_chans);
     if (!s->dry) {
       for (int b = 0; b < 2; ++b) {
         const uint8_t* x = q.has_turn ? s->base + q.off_turn : s->base + q.off_in[b];
@@ -387,16 +390,16 @@ int corr_svc_tick(corr_svc* s, int* n_requests) {
       I.vec_ok = 1;
       s->h_tmaps[p][inst] = q->tmap[b];
     }
-    // one launch per (sample width, nibble order, payload order read directly);
-    // tasks longest first
-    struct Cls { int bits, lo; bool tci; std::vector<Req*> qs; };
+    // one launch per (sample width, nibble order, payload order read directly,
+    // pairs of CTAs); tasks longest first
+    struct Cls { int bits, lo; bool tci, pair; std::vector<Req*> qs; };
     std::vector<Cls> cls;
     for (Req* q : parts) {
       const int lo = (q->r.flags & CORR_F_LO_IS_REAL) ? 1 : 0;
       auto c = std::find_if(cls.begin(), cls.end(), [&](const Cls& x) {
-        return x.bits == q->r.bits && x.lo == lo && x.tci == q->tci;
+        return x.bits == q->r.bits && x.lo == lo && x.tci == q->tci && x.pair == q->pair;
       });
-      if (c == cls.end()) cls.push_back({q->r.bits, lo, q->tci, {q}});
+      if (c == cls.end()) cls.push_back({q->r.bits, lo, q->tci, q->pair, {q}});
       else c->qs.push_back(q);
     }
     size_t ntask = 0;
@@ -406,7 +409,7 @@ int corr_svc_tick(corr_svc* s, int* n_requests) {
     if (!ensure(s->d_tasks[p], s->h_tasks[p], s->task_cap[p], ntask) ||
         !ensure(s->d_first[p], s->h_first[p], s->first_cap[p], cls.size() * (nsm + 1)))
       return CORR_ENOMEM;
-    struct Launch { size_t t0, f0; int nt, nc, bits, lo; bool tci; };
+    struct Launch { size_t t0, f0; int nt, nc, bits, lo; bool tci, pair; };  // nc: CTAs, or pairs
     std::vector<Launch> ls;
     size_t tpos = 0, fpos = 0;
     for (auto& c : cls) {
@@ -419,15 +422,17 @@ int corr_svc_tick(corr_svc* s, int* n_requests) {
           const int nb = t.cb[1] >= 0 ? 2 : 1;
           const bool a_in = t.rb == t.cb[0] || (nb == 2 && t.rb == t.cb[1]);
           const int st = herk_ring_stage(q->r.bits);
-          cost.push_back((double)((q->r.block_spectra + st - 1) / st) * (a_in ? nb : nb + 1));
+          // (a pair's diagonal task: 2/3 of the shared-memory traffic of another)
+          cost.push_back((double)((q->r.block_spectra + st - 1) / st) *
+                         (c.pair ? (t.rb == t.cb[0] ? 2 : 3) : a_in ? nb : nb + 1));
           all.push_back(t);
         }
       }
-      const int nt = (int)all.size(), nc = std::min(nt, nsm);
+      const int nt = (int)all.size(), nc = std::min(nt, c.pair ? nsm / 2 : nsm);
       std::vector<int> order(nt);
       corr_plan_schedule(cost.data(), nt, nc, order.data(), s->h_first[p] + fpos);
       for (int j = 0; j < nt; ++j) s->h_tasks[p][tpos + j] = all[order[j]];
-      ls.push_back({tpos, fpos, nt, nc, c.bits, c.lo, c.tci});
+      ls.push_back({tpos, fpos, nt, nc, c.bits, c.lo, c.tci, c.pair});
       tpos += nt;
       fpos += nc + 1;
     }
@@ -451,7 +456,8 @@ int corr_svc_tick(corr_svc* s, int* n_requests) {
       a.lo_is_real = l.lo;
       a.bits = l.bits;
       a.n_tasks = l.nt;
-      a.grid = l.nc;
+      a.pair = l.pair ? 1 : 0;
+      a.grid = l.pair ? 2 * l.nc : l.nc;
       a.scratch = s->scratch;
       a.scratch_ctas = s->scratch_ctas;
       if (herk4_launch(a, nullptr, l.nt, s->stream, l.tci) != cudaSuccess) return CORR_ECUDA;
