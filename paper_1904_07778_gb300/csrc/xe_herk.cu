@@ -566,21 +566,25 @@ static_assert(kGroupThreads == 128, "an unpack group covers a packed block in fo
 constexpr int kMmaWarp = kUnpackWarps, kTmaWarp = kUnpackWarps + 1, kEpiWarp0 = kUnpackWarps + 4;
 constexpr int kEpiWarps = XE_EPI_WARPS;
 constexpr int kRingThreads = (kEpiWarp0 + kEpiWarps) * 32;
-// registers per thread: launch share, unpack warpgroups, the other warpgroups.
-// Chosen per instance from the compiler's spill report and measured times:
-// the 8-bit drain, which adds the accumulations' partial sums, takes more,
-// the 8-bit unpack less; the 4-bit unpack spills below 88 (the cylinder block
-// 1.11 ms at 80 / 56 against 1.07).
+// registers per thread: launch share, unpack warpgroups, the loader's and MMA
+// issuer's warpgroup, drain warpgroups.  Chosen per instance from the
+// compiler's spill report and measured times: the 8-bit drain, which adds the
+// accumulations' partial sums, takes more, the 8-bit unpack less; the 4-bit
+// unpack spills below 88 (the cylinder block 1.11 ms at 80 / 56 against 1.07).
+// The loader and the issuer need no more than 40, which leaves the 4-bit drain
+// 56 instead of 48: push and dump of 192 x 1024 inputs x channels, 137 -> 133
+// us at 1024 spectra and 116 -> 111 at 512.
 constexpr int kRegsLaunch = (65536 / kRingThreads) & ~7;
 template <bool LO, bool EIGHT>
 __host__ __device__ constexpr int regs_unpack() { return EIGHT ? 72 : 88; }
-template <bool LO, bool EIGHT>
-__host__ __device__ constexpr int regs_other() { return EIGHT ? 72 : 48; }
+constexpr int kRegsMma = 40;
+template <bool EIGHT>
+__host__ __device__ constexpr int regs_drain() { return EIGHT ? 88 : 56; }
 static_assert(kRingThreads % 128 == 0, "whole warpgroups");
 template <bool LO, bool EIGHT>
 constexpr bool regs_fit() {
   return kUnpackWarps * 32 * regs_unpack<LO, EIGHT>() +
-             (kRingThreads - kUnpackWarps * 32) * regs_other<LO, EIGHT>() <=
+             (kEpiWarp0 - kUnpackWarps) * 32 * kRegsMma + kEpiWarps * 32 * regs_drain<EIGHT>() <=
          kRingThreads * kRegsLaunch;
 }
 static_assert(regs_fit<false, false>() && regs_fit<true, false>() && regs_fit<false, true>(),
@@ -733,7 +737,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
   // joined again would leave the compiler the smaller budget for all roles.
   if (warp == kTmaWarp) {
     // ------------------------------------------------------------ TMA loader
-    regs_shrink<regs_other<LO_IS_REAL, EIGHT>()>();
+    regs_shrink<kRegsMma>();
     if (lane == 0 && n_my > 0) {
       if (!a.tmaps) tma_prefetch_desc(&tmap);
       // fault injection: this stage of CTA 0 is never loaded, so the waits
@@ -793,7 +797,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
     __syncwarp();
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------------ MMA issuer
-    regs_shrink<regs_other<LO_IS_REAL, EIGHT>()>();
+    regs_shrink<kRegsMma>();
     if (lane == 0 && rank == 0) {  // (a pair's MMAs are all issued by CTA 0)
       int s = 0, m = 0, v = 0;  // v: accumulations so far (tensor-memory buffer v & 1)
       bool ok = true;
@@ -1066,10 +1070,13 @@ __global__ void __launch_bounds__(kRingThreads, 1)
     }
     if (EIGHT && __any_sync(0xFFFFFFFFu, bad != 0) && lane == 0) raise_status(a, kStRange);
   } else if (warp < kEpiWarp0) {
-    regs_shrink<regs_other<LO_IS_REAL, EIGHT>()>();  // the two idle warps of the MMA / TMA warpgroup
+    regs_shrink<kRegsMma>();  // the two idle warps of the MMA / TMA warpgroup
   } else {
     // ------------------------------------------------------------ drain
-    regs_shrink<regs_other<LO_IS_REAL, EIGHT>()>();
+    if constexpr (regs_drain<EIGHT>() > kRegsLaunch)
+      regs_grow<regs_drain<EIGHT>()>();
+    else
+      regs_shrink<regs_drain<EIGHT>()>();
     const int quad = warp & 3, part = (warp - kEpiWarp0) >> 2;
     int2* scr = EIGHT ? a.scratch + (size_t)blockIdx.x * kHerkScratchInt2 : nullptr;
     int v = 0;
