@@ -432,50 +432,103 @@ __global__ void pad_rows_kernel(const uint8_t* __restrict__ in, uint8_t* __restr
 // ---------------------------------------------------------------- normalise
 // rho = V / sqrt(V_ii V_jj) for a range of one channel's baselines.
 //
-// Bound: the FP64 pipe, which on this chip is 80 times narrower than FP32
-// (1.59 FMAs a cycle per SM, measured), far ahead of the 32 bytes a baseline
-// moves.  So the square root and the two divisions of a baseline are not
-// called.  A block keeps 1 / sqrt(V_ii) and sqrt(V_ii) of its channel's inputs
-// in shared memory (one rsqrt per input, not per baseline) as float pairs;
-// their products, and those with V's parts, give the reciprocal of the
-// denominator, the denominator and the quotients to about 2^-46 in FP32 and
-// integer operations; and one FMA residual step each, exact to well below the
-// last bit, rounds the square root and the quotients as sqrt and / do
-// (Markstein's correction: s + (x - s^2) y / 2 and q + (a - q d) y; compared
-// with sqrt and / over 3e9 random operands without a difference).  That
-// leaves 7 FP64 operations a baseline, 0.27 ms of the pipe for 192 inputs x
-// 1024 channels: the call takes 345 us, 471 us with the estimates in FP64
-// too (11 operations), 1700 us with sqrt and two divisions.  The baseline's
-// inputs come from an FP32 square root and integers.
+// The FP64 pipe is 80 times narrower on this chip than FP32 (1.59 FMAs a cycle
+// per SM, measured), and a square root and two divisions on it cost a baseline
+// far more than its 32 bytes.  So both are made from float pairs and integers.
+// A block keeps 1 / sqrt(V_ii) and sqrt(V_ii) of its channel's inputs in shared
+// memory (one rsqrt per input, not per baseline) as float pairs.  Their
+// products, and those with V's parts, give the 53-bit significands of the
+// denominator and of the quotients to about 2^-45.  The remainders
+// D - s^2 and a - q s are then below 2^63 and exact in the low 64 bits of
+// integer products; they give the correction to within half a unit and a
+// little, and the new remainder's sign against half a unit the last step.  So
+// the results are those of sqrt and / (also compared over 10^9 random
+// operands, without a difference).  One FP64 product a baseline is left, the
+// denominator's square.
+// The call (192 inputs x 1024 channels): KNOW us; 345 with the roundings by
+// FP64 residuals (7 operations of that pipe), 471 with the estimates in FP64
+// too (11), 1700 with sqrt and two divisions.
 constexpr int kNormThreads = 256;
 
-// (double)v without the FP64 pipe (the conversion instruction costs about
-// three of its operations): exact for |v| < 2^31 in integer operations.
-__device__ __forceinline__ double s64_to_double(long long v) {
-  const int x = (int)v;
-  if (v != (long long)x || x == (int)0x80000000) return (double)v;
-  const uint32_t u = (uint32_t)abs(x);
-  if (u == 0) return 0.0;
-  const int z = __clz((int)u);
-  const uint32_t m = u << z;  // 1.f in bits 31..0
-  // exponent 1023 + 31 - z; the leading one of m adds the missing exponent step
-  const uint32_t hi = ((uint32_t)x & 0x80000000u) + ((uint32_t)(1053 - z) << 20) + (m >> 11);
-  return __hiloint2double((int)hi, (int)(m << 21));
+// A correctly rounded square root: m 2^(e - 52), m in [2^52, 2^53), and
+// 2^e over it as a float pair, good to 2^-45.
+struct NormRoot {
+  uint64_t m;
+  int e;
+  float yh, yl;
+};
+
+// The significand h + l, a float pair in units of its last bit over 2^28, as an integer.
+__device__ __forceinline__ uint64_t sig_of(float h, float l) {
+  return ((uint64_t)(long long)__float2int_rn(h) << 28) + 2 * (long long)__float2int_rn(l * 134217728.0f);
+}
+__device__ __forceinline__ int small_rn(float c) {  // |c| < 2^22
+  return (int)(__float_as_uint(c + 12582912.0f) - 0x4B400000u);
 }
 
-// The float pair a + b (|b| well below |a|; a normal, at least 2^-75 in
-// magnitude) as a double, in integers: the pair is renormalised (fast
-// two-sum), and its low part, in units of the high part's double ulp, is added
-// to the high part's widened bits.
-__device__ __forceinline__ double widen(float a, float b) {
-  const float h = a + b, e = b - (h - a);  // |e| <= half an ulp of h
-  const uint32_t u = __float_as_uint(h) & 0x7FFFFFFFu;
-  const float ulps = __uint_as_float((306u - (u >> 23)) << 23);  // 2^52 over h's power of two
-  int i = __float2int_rn(e * ulps);
-  if (h < 0.f) i = -i;
-  if ((u << 9) == 0 && i < 0) i *= 2;  // h a power of two: the ulp below it is half
-  const long long d = ((long long)u << 29) + (896ll << 52) + i;
-  return __longlong_as_double(d | ((long long)(__float_as_uint(h) & 0x80000000u) << 32));
+// sqrt(den2), den2 >= 1, from the pairs of 1 / sqrt(den2) and sqrt(den2).
+__device__ __forceinline__ NormRoot norm_root(double den2, float yh, float yl, float sh, float sl) {
+  const uint64_t d = (uint64_t)__double_as_longlong(den2);
+  const int x = (int)(d >> 52) - 1023;
+  NormRoot r;
+  r.e = x >> 1;
+  const float up = __uint_as_float((uint32_t)(127 + r.e) << 23);
+  const float dn = __uint_as_float((uint32_t)(151 - r.e) << 23);  // 2^24 over it
+  r.yh = yh * up;
+  r.yl = yl * up;
+  uint64_t m = sig_of(sh * dn, sl * dn);
+  // den2 is n 2^(2 e - 104), n an integer of up to 106 bits: its low 64 are the
+  // last 12 of den2's significand (doubled for odd exponents)
+  long long rem = (long long)((d << (52 + (x & 1))) - m * m);
+  const int k = small_rn((float)(int)(rem >> 32) * (r.yh * 0x1p-21f));
+  rem -= (long long)((uint64_t)(long long)k * (2 * m + (uint64_t)(long long)k));
+  m += (uint64_t)(long long)k;
+  // (m +- 1/2)^2 = m^2 +- m + 1/4
+  if (rem > (long long)m)
+    ++m;
+  else if (rem <= -(long long)m)
+    --m;
+  r.m = m;
+  return r;
+}
+
+// w over the root, correctly rounded.
+__device__ __forceinline__ double norm_divide(long long w, const NormRoot& r) {
+  uint64_t a;  // |w| 2^(53 - bits), in [2^52, 2^53)
+  int bits;
+  const int w32 = (int)w;
+  if (w == (long long)w32 && w32 != (int)0x80000000) {
+    const uint32_t u = (uint32_t)abs(w32);
+    if (u == 0) return 0.0;
+    const int z = __clz((int)u);
+    a = (uint64_t)(u << z) << 21;
+    bits = 32 - z;
+  } else {
+    const uint64_t u = (uint64_t)llabs(w);
+    if (u >> 53)  // rounded to a double first
+      return (double)w / __longlong_as_double((long long)(((uint64_t)(r.e + 1022) << 52) + r.m));
+    const int z = __clzll((long long)u);
+    a = u << z >> 11;
+    bits = 64 - z;
+  }
+  // its first 24 bits as a float in [1, 2), and the next 23
+  const float ah = __uint_as_float((uint32_t)(a >> 29) + 0x3F000000u);
+  const float al = (__uint_as_float(((uint32_t)a << 3 >> 9) | 0x3F800000u) - 1.0f) * 0x1p-23f;
+  const bool big = a >= r.m;  // the quotient of the significands is at least 1
+  const float scale = big ? 0x1p24f : 0x1p25f;
+  const float qh = ah * r.yh, ql = fmaf(al, r.yh, fmaf(ah, r.yl, fmaf(ah, r.yh, -qh)));
+  uint64_t q = sig_of(qh * scale, ql * scale);
+  long long rem = (long long)((a << (big ? 52 : 53)) - q * r.m);
+  const int k = small_rn((float)(int)(rem >> 32) * (r.yh * 0x1p-20f));
+  rem -= (long long)((uint64_t)(long long)k * r.m);
+  q += (uint64_t)(long long)k;
+  if (2 * rem > (long long)r.m)
+    ++q;
+  else if (2 * rem < -(long long)r.m)
+    --q;
+  const int x = bits - 1 - r.e - (big ? 0 : 1);
+  const uint64_t v = ((uint64_t)(x + 1022) << 52) + q;
+  return __longlong_as_double((long long)(v | ((uint64_t)w & 0x8000000000000000ull)));
 }
 
 // An input's factors: the power V_ii, and 1 / sqrt(V_ii) and sqrt(V_ii) as
@@ -525,30 +578,14 @@ __global__ void __launch_bounds__(kNormThreads)
     double re = 0.0, im = 0.0;
     const int top = __double2hiint(den2);  // |den2| is 0 or at least 1: its sign and zero from the high word
     if (top > 0) {
-      // 1 / sqrt(den2) and sqrt(den2) to about 2^-46, as float pairs
+      // 1 / sqrt(den2) and sqrt(den2) as float pairs
       const float yh = ni.yh * nj.yh;
       const float yl = fmaf(ni.yl, nj.yh, fmaf(ni.yh, nj.yl, fmaf(ni.yh, nj.yh, -yh)));
       const float sh = ni.rh * nj.rh;
       const float sl = fmaf(ni.rl, nj.rh, fmaf(ni.rh, nj.rl, fmaf(ni.rh, nj.rh, -sh)));
-      const double y = widen(yh, yl), s = widen(sh, sl);
-      // y / 2: one off the exponent (y is a normal number: powers are >= 1)
-      const double h = __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y));
-      const double den = fma(fma(-s, s, den2), h, s);
-      auto divide = [&](long long w) {
-        const int x = (int)w;
-        double q;
-        if (w == (long long)x && abs(x) < (1 << 30)) {
-          if (x == 0) return 0.0;
-          const float xh = (float)x, xl = (float)(x - __float2int_rn(xh));
-          const float qh = xh * yh;
-          q = widen(qh, fmaf(xl, yh, fmaf(xh, yl, fmaf(xh, yh, -qh))));
-        } else {
-          q = (double)w * y;
-        }
-        return fma(fma(-q, den, s64_to_double(w)), y, q);
-      };
-      re = divide(vr);
-      im = divide(vi);
+      const NormRoot root = norm_root(den2, yh, yl, sh, sl);
+      re = norm_divide(vr, root);
+      im = norm_divide(vi, root);
     } else if ((top << 1) != 0) {
       re = im = sqrt(den2);  // not a power: NaN
     }
