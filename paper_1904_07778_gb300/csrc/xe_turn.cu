@@ -436,7 +436,7 @@ __global__ void pad_rows_kernel(const uint8_t* __restrict__ in, uint8_t* __restr
 // per SM, measured), and a square root and two divisions on it cost a baseline
 // far more than its 32 bytes.  So both are made from float pairs and integers.
 // A block keeps 1 / sqrt(V_ii) and sqrt(V_ii) of its channel's inputs in shared
-// memory (one rsqrt per input, not per baseline) as float pairs.  Their
+// memory (one root per input, not per baseline) as float pairs.  Their
 // products, and those with V's parts, give the 53-bit significands of the
 // denominator and of the quotients to about 2^-45.  The remainders
 // D - s^2 and a - q s are then below 2^63 and exact in the low 64 bits of
@@ -444,10 +444,11 @@ __global__ void pad_rows_kernel(const uint8_t* __restrict__ in, uint8_t* __restr
 // little, and the new remainder's sign against half a unit the last step.  So
 // the results are those of sqrt and / (also compared over 10^9 random
 // operands, without a difference).  One FP64 product a baseline is left, the
-// denominator's square.
-// The call (192 inputs x 1024 channels): KNOW us; 345 with the roundings by
+// denominator's square.  What bounds it now is the issue of some 230
+// instructions a baseline (74% of the slots), then the 32 bytes (0.09 ms).
+// The call (192 inputs x 1024 channels): 163 us; 345 with the roundings by
 // FP64 residuals (7 operations of that pipe), 471 with the estimates in FP64
-// too (11), 1700 with sqrt and two divisions.
+// too (11), 1700 with sqrt and two divisions.  64 x 512: 25 us.
 constexpr int kNormThreads = 256;
 
 // A correctly rounded square root: m 2^(e - 52), m in [2^52, 2^53), and
@@ -460,75 +461,87 @@ struct NormRoot {
 
 // The significand h + l, a float pair in units of its last bit over 2^28, as an integer.
 __device__ __forceinline__ uint64_t sig_of(float h, float l) {
-  return ((uint64_t)(long long)__float2int_rn(h) << 28) + 2 * (long long)__float2int_rn(l * 134217728.0f);
+  return (uint64_t)(uint32_t)__float2int_rn(h) * (1u << 28) + (uint64_t)(2ll * __float2int_rn(l * 134217728.0f));
 }
-__device__ __forceinline__ int small_rn(float c) {  // |c| < 2^22
-  return (int)(__float_as_uint(c + 12582912.0f) - 0x4B400000u);
+// Bits 32 .. 63 of p q.
+__device__ __forceinline__ uint32_t product_word1(uint64_t p, uint64_t q) {
+  const uint32_t pl = (uint32_t)p, ph = (uint32_t)(p >> 32), ql = (uint32_t)q, qh = (uint32_t)(q >> 32);
+  return __umulhi(pl, ql) + pl * qh + ph * ql;
+}
+// A correction of c units, |c| < 2^10 and good to 2^-13, as an integer k; near
+// says that c is too close to half a unit for its nearest integer to be sure.
+__device__ __forceinline__ int nearest(float c, bool& near) {
+  const float t = c + 12582912.0f;  // 1.5 2^23
+  near = fabsf(c - (t - 12582912.0f)) > 0.499f;
+  return (int)(__float_as_uint(t) - 0x4B400000u);
 }
 
 // sqrt(den2), den2 >= 1, from the pairs of 1 / sqrt(den2) and sqrt(den2).
 __device__ __forceinline__ NormRoot norm_root(double den2, float yh, float yl, float sh, float sl) {
-  const uint64_t d = (uint64_t)__double_as_longlong(den2);
-  const int x = (int)(d >> 52) - 1023;
+  const uint32_t hi = (uint32_t)__double2hiint(den2), lo = (uint32_t)__double2loint(den2);
+  const int x = (int)(hi >> 20) - 1023;
   NormRoot r;
   r.e = x >> 1;
   const float up = __uint_as_float((uint32_t)(127 + r.e) << 23);
   const float dn = __uint_as_float((uint32_t)(151 - r.e) << 23);  // 2^24 over it
   r.yh = yh * up;
   r.yl = yl * up;
-  uint64_t m = sig_of(sh * dn, sl * dn);
+  const uint64_t m = sig_of(sh * dn, sl * dn);
   // den2 is n 2^(2 e - 104), n an integer of up to 106 bits: its low 64 are the
   // last 12 of den2's significand (doubled for odd exponents)
-  long long rem = (long long)((d << (52 + (x & 1))) - m * m);
-  const int k = small_rn((float)(int)(rem >> 32) * (r.yh * 0x1p-21f));
-  rem -= (long long)((uint64_t)(long long)k * (2 * m + (uint64_t)(long long)k));
-  m += (uint64_t)(long long)k;
-  // (m +- 1/2)^2 = m^2 +- m + 1/4
-  if (rem > (long long)m)
-    ++m;
-  else if (rem <= -(long long)m)
-    --m;
-  r.m = m;
+  const uint32_t n1 = lo << (20 + (x & 1));
+  bool near;
+  const int k = nearest((float)(int)(n1 - product_word1(m, m)) * (r.yh * 0x1p-21f), near);
+  r.m = m + (uint64_t)(long long)k;
+  if (near) {  // (m +- 1/2)^2 = m^2 +- m + 1/4
+    const long long rem = (long long)(((uint64_t)n1 << 32) - r.m * r.m), mk = (long long)r.m;
+    r.m += rem > mk ? 1 : rem <= -mk ? -1 : 0;
+  }
   return r;
 }
 
-// w over the root, correctly rounded.
-__device__ __forceinline__ double norm_divide(long long w, const NormRoot& r) {
-  uint64_t a;  // |w| 2^(53 - bits), in [2^52, 2^53)
-  int bits;
-  const int w32 = (int)w;
-  if (w == (long long)w32 && w32 != (int)0x80000000) {
-    const uint32_t u = (uint32_t)abs(w32);
-    if (u == 0) return 0.0;
-    const int z = __clz((int)u);
-    a = (uint64_t)(u << z) << 21;
-    bits = 32 - z;
-  } else {
-    const uint64_t u = (uint64_t)llabs(w);
-    if (u >> 53)  // rounded to a double first
-      return (double)w / __longlong_as_double((long long)(((uint64_t)(r.e + 1022) << 52) + r.m));
-    const int z = __clzll((long long)u);
-    a = u << z >> 11;
-    bits = 64 - z;
-  }
-  // its first 24 bits as a float in [1, 2), and the next 23
-  const float ah = __uint_as_float((uint32_t)(a >> 29) + 0x3F000000u);
-  const float al = (__uint_as_float(((uint32_t)a << 3 >> 9) | 0x3F800000u) - 1.0f) * 0x1p-23f;
+// a over the root's significand, a = |w| 2^(53 - bits) in [2^52, 2^53) and ah +
+// al its leading bits as a float pair in [1, 2): the quotient, correctly
+// rounded, with w's sign.
+__device__ __forceinline__ double norm_quotient(uint64_t a, float ah, float al, int bits, uint32_t sign,
+                                                const NormRoot& r) {
   const bool big = a >= r.m;  // the quotient of the significands is at least 1
   const float scale = big ? 0x1p24f : 0x1p25f;
   const float qh = ah * r.yh, ql = fmaf(al, r.yh, fmaf(ah, r.yl, fmaf(ah, r.yh, -qh)));
   uint64_t q = sig_of(qh * scale, ql * scale);
-  long long rem = (long long)((a << (big ? 52 : 53)) - q * r.m);
-  const int k = small_rn((float)(int)(rem >> 32) * (r.yh * 0x1p-20f));
-  rem -= (long long)((uint64_t)(long long)k * r.m);
+  const uint32_t a1 = (uint32_t)a << (big ? 20 : 21);  // bits 32 .. 63 of a 2^52, a 2^53
+  bool near;
+  const int k = nearest((float)(int)(a1 - product_word1(q, r.m)) * (r.yh * 0x1p-20f), near);
   q += (uint64_t)(long long)k;
-  if (2 * rem > (long long)r.m)
-    ++q;
-  else if (2 * rem < -(long long)r.m)
-    --q;
-  const int x = bits - 1 - r.e - (big ? 0 : 1);
-  const uint64_t v = ((uint64_t)(x + 1022) << 52) + q;
-  return __longlong_as_double((long long)(v | ((uint64_t)w & 0x8000000000000000ull)));
+  if (near) {
+    const long long rem = (long long)(((uint64_t)a1 << 32) - q * r.m);
+    q += 2 * rem > (long long)r.m ? 1 : 2 * rem < -(long long)r.m ? -1 : 0;
+  }
+  const uint32_t x = (uint32_t)(bits - 1 - r.e - (big ? 0 : 1) + 1022);
+  return __hiloint2double((int)((x << 20) + (uint32_t)(q >> 32) + (sign & 0x80000000u)), (int)(uint32_t)q);
+}
+
+__device__ __noinline__ double norm_divide_wide(long long w, const NormRoot r) {
+  const uint64_t u = (uint64_t)llabs(w);
+  if (u >> 53)  // rounded to a double first
+    return (double)w / __longlong_as_double((long long)(((uint64_t)(r.e + 1022) << 52) + r.m));
+  const int z = __clzll((long long)u);
+  const uint64_t a = u << z >> 11;
+  const float ah = __uint_as_float((uint32_t)(a >> 29) + 0x3F000000u);
+  const float al = (__uint_as_float(((uint32_t)a << 3 >> 9) | 0x3F800000u) - 1.0f) * 0x1p-23f;
+  return norm_quotient(a, ah, al, 64 - z, (uint32_t)(w >> 32), r);
+}
+// w over the root, correctly rounded.
+__device__ __forceinline__ double norm_divide(long long w, const NormRoot& r) {
+  const int x = (int)w;
+  if (w != (long long)x || x == (int)0x80000000) return norm_divide_wide(w, r);
+  const uint32_t u = (uint32_t)abs(x);
+  if (u == 0) return 0.0;
+  const int z = __clz((int)u);
+  const uint32_t t = u << z;
+  const float ah = __uint_as_float((t >> 8) + 0x3F000000u);
+  const float al = (__uint_as_float((t & 0xFFu) | 0x3F800000u) - 1.0f) * 0x1p-8f;
+  return norm_quotient((uint64_t)t * (1u << 21), ah, al, 32 - z, (uint32_t)x, r);
 }
 
 // An input's factors: the power V_ii, and 1 / sqrt(V_ii) and sqrt(V_ii) as
@@ -538,7 +551,7 @@ struct NormInput {
   float yh, yl, rh, rl;
 };
 
-__global__ void __launch_bounds__(kNormThreads)
+__global__ void __launch_bounds__(kNormThreads, 6)
     normalise_kernel(const int64_t* __restrict__ acc, double* __restrict__ rho,
                      uint8_t* __restrict__ zero_flag, int nbl, int per_block, int vec_ok) {
   extern __shared__ __align__(16) NormInput norm_sm[];
@@ -546,7 +559,8 @@ __global__ void __launch_bounds__(kNormThreads)
   const int b0 = blockIdx.x * per_block, b1 = min(nbl, b0 + per_block);
   const int64_t* v = acc + c * nbl * 2;
   auto input_of = [](int b) {  // i with i (i + 1) / 2 <= b < (i + 1) (i + 2) / 2; 8 b + 1 < 2^24
-    int i = (int)((sqrtf((float)(8 * b + 1)) - 1.0f) * 0.5f);
+    const float x = (float)(8 * b + 1);
+    int i = (int)((x * rsqrtf(x) - 1.0f) * 0.5f);  // within one
     if (i * (i + 1) / 2 > b) --i;
     if ((i + 1) * (i + 2) / 2 <= b) ++i;
     return i;
@@ -554,17 +568,24 @@ __global__ void __launch_bounds__(kNormThreads)
   const int last = input_of(b1 - 1);  // no baseline of the range has a larger input
   for (int i = threadIdx.x; i <= last; i += kNormThreads) {
     NormInput n;
-    n.p = (double)v[i * (i + 3)];
-    const double y = rsqrt(fabs(n.p)), r = fabs(n.p) * y;
-    n.yh = (float)y;
-    n.yl = (float)(y - (double)n.yh);
-    n.rh = (float)r;
-    n.rl = (float)(r - (double)n.rh);
+    const long long p = v[i * (i + 3)];
+    n.p = (double)p;
+    // |p| as a float pair; a Newton step from the FP32 estimate, in pairs:
+    // y + y e / 2 + 3 y e^2 / 8 with e = 1 - p y^2
+    const float ph = (float)p, pl = (float)(p - (long long)ph), y = rsqrtf(fabsf(ph));
+    const float ah = fabsf(ph), al = ph < 0.f ? -pl : pl, t = y * y;
+    const float e = fmaf(-al, t, fmaf(-ah, fmaf(y, y, -t), fmaf(-ah, t, 1.0f)));
+    n.yh = y;
+    n.yl = y * fmaf(0.375f * e, e, 0.5f * e);
+    n.rh = ah * y;
+    n.rl = fmaf(al, y, fmaf(ah, n.yl, fmaf(ah, y, -n.rh)));
     norm_sm[i] = n;
   }
   __syncthreads();
-  for (int b = b0 + (int)threadIdx.x; b < b1; b += kNormThreads) {
-    const int i = input_of(b), j = b - i * (i + 1) / 2;
+  int i = input_of(b0 + (int)threadIdx.x), j = b0 + (int)threadIdx.x - i * (i + 1) / 2;
+  for (int b = b0 + (int)threadIdx.x; b < b1; b += kNormThreads, j += kNormThreads) {
+    for (; j > i; j -= ++i) {
+    }
     const long long e = c * nbl + b;
     long long vr, vi;
     if (vec_ok) {

@@ -48,3 +48,28 @@ def test_normalise_is_ieee(N, C, mag, skew):
     assert np.array_equal(flag.cpu().numpy().reshape(C, nbl), zf)
     rest = buf.cpu().numpy()
     assert (np.concatenate([rest[:skew], rest[skew + C * nbl * 2:]]) == 7.0).all()
+
+
+def test_normalise_at_the_edges():
+    """Powers and numerators where the significands change length: powers of
+    two and their neighbours, the ends of 32 and 53 bits and of the type."""
+    import torch
+    from paper_1904_07778_gb300 import xengine as xe
+    p = [1, 2, 3, (1 << 24) - 1, (1 << 24) + 1, (1 << 31) - 1, 1 << 31, (1 << 52) - 1, (1 << 53) - 1, (1 << 53) + 1,
+         (1 << 62), (1 << 63) - 1, 5, 1 << 40]
+    w = [1, 3, (1 << 24) - 1, (1 << 24) + 1, (1 << 31) - 1, 1 << 31, (1 << 31) + 1, (1 << 32) - 1, (1 << 53) - 1, 1 << 53,
+         (1 << 53) + 1, (1 << 63) - 1]
+    w = np.array([0, -(1 << 63)] + w + [-x for x in w], np.int64)
+    N, C = len(p), len(w)
+    vis = np.empty((C, N * (N + 1) // 2, 2), np.int64)
+    vis[..., 0] = w[:, None]
+    vis[..., 1] = np.roll(w, 5)[:, None]
+    d = np.arange(N) * (np.arange(N) + 3) // 2
+    vis[:, d, 0] = p
+    want, _ = _want(vis, N)
+    rho = torch.empty(vis.shape, dtype=torch.float64, device="cuda")
+    with xe.Correlator(N, C, 16, bits=4, layout=2) as cor:
+        cor.restore(vis)
+        cor.normalise_into(rho)
+        torch.cuda.synchronize()
+    assert np.array_equal(rho.cpu().numpy().view(np.int64), want.view(np.int64))
