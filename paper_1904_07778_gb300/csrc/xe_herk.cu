@@ -322,8 +322,9 @@ __device__ __forceinline__ void mma_loop(const TaskGeom& g, int nk, int nst, uin
 // Drain the accumulators, correct the offset codes (4-bit), fold 2 x 2 real
 // blocks into complex visibilities and store or add them into the int64
 // integration buffer.  The calling warp reads tensor-memory lanes
-// 32 quad .. + 31 (rows of the A block; quad must be the warp index mod 4)
-// and every nparts-th 16-column chunk from the part-th on.  Column block
+// 32 quad .. + 31 (rows of the A block; quad must be the warp index mod 4);
+// of nparts = 2 warps a quarter, part 0 and 1 take one 16-row half each with
+// HALVES, else alternate 16-column chunks of both.  Column block
 // c < rb is a lower-triangle block, c == rb the diagonal block (entries
 // j <= i only), c > rb the transpose of block (c, rb): there the thread's
 // row is the second input of the baseline and the imaginary part changes
@@ -343,8 +344,16 @@ __device__ __forceinline__ void mma_loop(const TaskGeom& g, int nk, int nst, uin
 // its own serial instructions, about 10 cycles each on the shared SMSPs, so
 // the walk along a row or column carries only a pointer and a limit.
 // Push and dump of 192 x 1024 x 1024 [c][i][t]: 0.179 -> 0.145 ms (0.141 with
-// the row sums' exchanges below); 16 dish blocks in one launch 0.504 -> 0.493
-// (0.484) ms.
+// the row sums' exchanges below, 0.133 with 56 registers, 0.124 with HALVES);
+// 16 dish blocks in one launch 0.504 -> 0.493 (0.484) ms.
+//
+// HALVES and ACC (1 adds to the buffer, 0 stores, -1 asks at run time): in the
+// 4-bit [c][row][t] kernels a half a warp, which halves the walks and their
+// set-up, and no test at each store: 192 x 1024 x 1024 133 -> 124 us, x 512
+// spectra 112 -> 101, 512 x 304 x 512 225 -> 203; 4096 and more spectra,
+// where the MMAs bound, within 0.5%.  The payload-order and 8-bit kernels keep
+// the short form: their unpack's code leaves no room for two drains (192 x
+// 1024 x 8192 622 -> 629, 32 inputs 480 -> 485).
 //
 // F16 (8-bit samples): the accumulators hold G itself.  A task is drained
 // once per accumulation of at most 1024 spectra; every accumulation but the
@@ -353,7 +362,7 @@ __device__ __forceinline__ void mma_loop(const TaskGeom& g, int nk, int nst, uin
 // by the same thread), which the next one adds in, and the last goes to the
 // integration buffer.  The int32 sums stay below 2 * 127^2 * 32768 < 2^31 for
 // the longest block.
-template <bool F16>
+template <bool F16, bool HALVES, int ACC>
 __device__ __forceinline__ void epilogue(const HerkInst& a, const HerkTask& task, const TaskGeom& g,
                                          const int32_t* usum, uint32_t tmem, int quad, int part,
                                          int nparts, int lane, bool first, bool last, int2* scr) {
@@ -361,8 +370,9 @@ __device__ __forceinline__ void epilogue(const HerkInst& a, const HerkTask& task
   const int half = a.rows_per_chan >> 1;  // samples per channel of a stacked tile (a power of two), 0: not stacked
   const int q0 = lane & 3;  // the thread's columns of each chunk: samples q0, q0 + 4
   const int nbl = n * (n + 1) / 2;  // below 2^30 (inputs <= 32768)
+  const int k0 = HALVES ? 0 : part, step = HALVES ? 1 : nparts;  // the warp's chunks
 #pragma unroll 1
-  for (int h = 0; h < 2; ++h) {  // the quarter's 16-row halves
+  for (int h = HALVES ? part : 0; h < 2; h += HALVES ? nparts : 1) {  // the quarter's 16-row halves
     const int gr = 2 * quad + h;            // the half's group of 8 samples
     const int m = 8 * gr + (lane >> 3) + (lane & 4);  // the thread's sample
     int ch = task.chan0, i = g.rb * 64 + m;
@@ -381,10 +391,11 @@ __device__ __forceinline__ void epilogue(const HerkInst& a, const HerkTask& task
     }
     const uint32_t trow = tmem + ((uint32_t)(quad * 32 + 16 * h) << 16);
     int4* const sp = reinterpret_cast<int4*>(scr) + (h * 4 + quad) * 32 + lane;
-    // Chunks c0 + k, c0 + k + nparts, ... below c0 + kn: emit(k, re0, im0,
+    // Chunks c0 + k0, c0 + k0 + step, ... below c0 + kn: emit(k, re0, im0,
     // re1, im1) takes the visibilities of columns 8 k + q0 and 8 k + q0 + 4.  A
     // chunk loads while the one before it is stored.
-    auto walk = [&](int c0, int k, int kn, auto&& emit) {
+    auto walk = [&](int c0, int kn, auto&& emit) {
+      int k = k0;
       if (k >= kn) return;
       uint32_t r[8];
       int4 prev = make_int4(0, 0, 0, 0);  // 8-bit: the sums of the pieces before
@@ -419,7 +430,7 @@ __device__ __forceinline__ void epilogue(const HerkInst& a, const HerkTask& task
           im1 = (int)(g10[1] - g01[1]);
         }
         const int kk = k;
-        k += nparts;
+        k += step;
         if (k < kn) {
           tmem_load_16x16(trow + (uint32_t)((c0 + k) * 16), r);
           if (F16 && !first) prev = sp[(c0 + k) * 256];
@@ -433,7 +444,7 @@ __device__ __forceinline__ void epilogue(const HerkInst& a, const HerkTask& task
     };
     auto put = [&](int64_t* p, int re, int im, bool ok) {
       if (!ok) return;
-      if (a.accumulate)
+      if (ACC < 0 ? a.accumulate : ACC)
         red_s64x2(p, re, im);  // at L2: nothing waits for the old value
       else
         st_s64x2(p, re, im);
@@ -442,7 +453,7 @@ __device__ __forceinline__ void epilogue(const HerkInst& a, const HerkTask& task
     auto row_walk = [&](int c0, int kn, int j0) {
       int64_t* const p = chp + 2 * (i * (i + 1) / 2 + j0 + q0);
       const int lim = i - j0 - q0;
-      walk(c0, part, kn, [&](int k, int re0, int im0, int re1, int im1) {
+      walk(c0, kn, [&](int k, int re0, int im0, int re1, int im1) {
         put(p + 16 * k, re0, im0, 8 * k <= lim);
         put(p + 16 * k + 8, re1, im1, 8 * k + 4 <= lim);
       });
@@ -453,7 +464,7 @@ __device__ __forceinline__ void epilogue(const HerkInst& a, const HerkTask& task
     } else if (half) {  // several channels in the rows' group: one chunk
       // a column and a row of the tile share a channel when their samples
       // agree above the samples-per-channel bits
-      walk(gr, part, 1, [&](int, int re0, int im0, int re1, int im1) {
+      walk(gr, 1, [&](int, int re0, int im0, int re1, int im1) {
         const int mc = 8 * gr + q0, j0 = mc & (half - 1), j1 = (mc + 4) & (half - 1);
         put(chp + 2 * (i * (i + 1) / 2 + j0), re0, im0, (mc ^ m) < half && j0 <= i);
         put(chp + 2 * (i * (i + 1) / 2 + j1), re1, im1, ((mc + 4) ^ m) < half && j1 <= i);
@@ -466,7 +477,7 @@ __device__ __forceinline__ void epilogue(const HerkInst& a, const HerkTask& task
           row_walk(8 * s, cblk == g.rb ? gr + 1 : 8, 64 * cblk);
         } else {  // baselines (j, i), j > i: the conjugate
           const int jb = 64 * cblk + q0;
-          walk(8 * s, part, 8, [&](int k, int re0, int im0, int re1, int im1) {
+          walk(8 * s, 8, [&](int k, int re0, int im0, int re1, int im1) {
             const int j = jb + 8 * k;
             int64_t* p = chp + 2 * (j * (j + 1) / 2 + i);
             put(p, re0, -im0, i >= 0 && j < n);
@@ -1097,8 +1108,17 @@ __global__ void __launch_bounds__(kRingThreads, 1)
           break;
         }
         tc_after_sync();
-        epilogue<EIGHT>(in, task, g, sm.usum[b], tmem + (uint32_t)(b * 256), quad, part,
-                        kEpiWarps / 4, lane, q == 0, q == np - 1, scr);
+        auto drain = [&](auto ACC) {
+          epilogue<EIGHT, !TCI && !EIGHT, decltype(ACC)::value>(in, task, g, sm.usum[b],
+                                                               tmem + (uint32_t)(b * 256), quad, part,
+                                                               kEpiWarps / 4, lane, q == 0, q == np - 1, scr);
+        };
+        if constexpr (TCI || EIGHT)
+          drain(std::integral_constant<int, -1>{});
+        else if (in.accumulate)
+          drain(std::integral_constant<int, 1>{});
+        else
+          drain(std::integral_constant<int, 0>{});
         tc_before_sync();
         __syncwarp();
         if (lane == 0) {
@@ -1252,7 +1272,7 @@ __global__ void __launch_bounds__(kLdgThreads, 1) herk4_ldg_kernel(const HerkArg
     if (!good && lane == 0) raise_timeout(args, abort);
     tc_after_sync();
     if (good && !*abort)
-      epilogue<false>(a, task, g, sm.usum, tmem, warp & 3, 0, 1, lane, true, true, nullptr);
+      epilogue<false, false, -1>(a, task, g, sm.usum, tmem, warp & 3, 0, 1, lane, true, true, nullptr);
   }
   tc_before_sync();
   __syncthreads();
