@@ -321,8 +321,8 @@ __device__ __forceinline__ float clamp18(uint32_t bits) {
 // With a gain of kWideGain or more, everything beyond the 18-bit range
 // saturates (2^17 * 120 = 7.5 2^21), and so does all that lies past w: the
 // spectra need no clamp before they are rounded, only the code does.  (A
-// spectrum stays below 2^21: M/2 127 sum |h| < 2^21, so v g 2^-21 < 2^18 and
-// both magic roundings keep exact.)
+// spectrum stays below 2^21: 128 sum |h| is at most 0.43 2^21, at 4096 samples
+// and 16 taps, so v g 2^-21 < 2^18 and both magic roundings keep exact.)
 constexpr uint32_t kWideGain = 120;
 // A rounded code (the bits of 1.5 2^23 + q) clamped from below, to -7; s4_pack
 // then saturates it from above.
@@ -340,6 +340,11 @@ __device__ __forceinline__ uint32_t s4_pack(int hi, int lo, uint32_t low) {
 __device__ __forceinline__ int round18(float x) {
   const float c = fminf(fmaxf(x, -131072.0f), 131071.0f);
   return __float_as_int(c + 12582912.0f) - 0x4B400000;
+}
+// The same from a rounded spectrum's bits (those of 1.5 2^23 + its integer; a
+// spectrum stays below 2^21, see kWideGain): two integer instructions.
+__device__ __forceinline__ int value18(uint32_t bits) {
+  return min(__viaddmax_s32((int)bits, -0x4B400000, -131072), 131071);
 }
 
 // Bytes r and r + 1 of w (biased: w holds x ^ 0x80 per byte, x the int8 sample)
@@ -379,7 +384,12 @@ __host__ __device__ constexpr int fe_min_blocks(int logm) { return logm <= 11 ? 
 // 1.78; the last pass and the separation in registers 1.59; classes within
 // warps 1.56; instances for up to four taps 1.55; the code clamped instead of
 // the spectra 1.52.
-// POWER: accumulate Eq. 3's power sums.  FRAMED: at most four taps and
+// POWER: accumulate Eq. 3's power sums, of 18-bit values clamped as integers
+// beside the equaliser's own rounding, joined over a CTA's units before they
+// are added to the caller's: ADC samples to visibilities and powers of 32 inputs
+// x 256 channels x 4096 spectra 201 -> 174 us, 192 x 512 x 2048 1123 -> 929 (with
+// the spectra clamped for both in floats, and every unit's sums added globally,
+// before).  FRAMED: at most four taps and
 // aligned frames, coefficients and frames in registers; otherwise any taps and
 // alignment.  (Instances of their own, so that each keeps the others'
 // registers free.)
@@ -599,7 +609,18 @@ __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine
         }
         const float2 gk = gains[k * NT];
         uint32_t q[2][2][2];  // [re, im][input][spectrum]: the bits of 1.5 2^23 + code
-        if (POWER || !wide) {
+        if constexpr (POWER) {  // Eq. 3's sums of the 18-bit values, clamped as integers
+#pragma unroll
+          for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+              const uint64_t r = p_add(X[j][c], magic);
+              const int v0 = value18((uint32_t)r), v1 = value18((uint32_t)(r >> 32));
+              pw[k][j] += (unsigned long long)((long long)v0 * v0);
+              if (n_act > 1) pw[k][j] += (unsigned long long)((long long)v1 * v1);
+            }
+        }
+        if (!wide) {
           const uint32_t bound = bounds[k * NT];
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
@@ -609,23 +630,10 @@ __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine
             for (int c = 0; c < 2; ++c) {
               float x0, x1;
               p_unpack(X[j][c], x0, x1);
-              uint64_t f;  // the rounded spectrum, clamped to the bound
-              if constexpr (POWER) {  // the 18-bit value first, for the sums
-                const uint64_t v18 = p_add(p_pack(fminf(fmaxf(x0, -131072.0f), 131071.0f),
-                                                  fminf(fmaxf(x1, -131072.0f), 131071.0f)), magic);
-                const int v0 = (int)(uint32_t)v18 - 0x4B400000, v1 = (int)(uint32_t)(v18 >> 32) - 0x4B400000;
-                pw[k][j] += (unsigned long long)((long long)v0 * v0);
-                if (n_act > 1) pw[k][j] += (unsigned long long)((long long)v1 * v1);
-                f = p_sub(v18, magic);
-                if (!wide) {
-                  p_unpack(f, x0, x1);
-                  const float w = __uint_as_float(wb);
-                  f = p_pack(fminf(fmaxf(x0, -w), w), fminf(fmaxf(x1, -w), w));
-                }
-              } else {
-                const float hi = clamp18(wb), lo = -(hi + kClampSkew);
-                f = p_sub(p_add(p_pack(fminf(fmaxf(x0, lo), hi), fminf(fmaxf(x1, lo), hi)), magic), magic);
-              }
+              // the rounded spectrum, clamped to the bound
+              const float hi = clamp18(wb), lo = -(hi + kClampSkew);
+              const uint64_t f =
+                  p_sub(p_add(p_pack(fminf(fmaxf(x0, lo), hi), fminf(fmaxf(x1, lo), hi)), magic), magic);
               const uint64_t e = p_fma(f, g, magic);
               q[c][j][0] = (uint32_t)e;
               q[c][j][1] = (uint32_t)(e >> 32);
@@ -709,12 +717,21 @@ __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine
   }
 
   if constexpr (POWER) {
+    // the units of a CTA have the same channels: their sums meet in shared memory
+    // (z is free), and one unit's threads add them to the caller's
+    unsigned long long* const sums = reinterpret_cast<unsigned long long*>(fe_smem);  // [q][unit][lt]
+    if constexpr (U > 1) {
+      __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int nu = channel(k);
-      // every unit of the CTA summed its own spectra: add them all
-      atomicAdd(a.power + (long long)nu * N + i0, pw[k][0]);
-      if (has1) atomicAdd(a.power + (long long)nu * N + i0 + 1, pw[k][1]);
+      for (int q = 0; q < 8; ++q) sums[q * NT + tid] = pw[q >> 1][q & 1];
+      __syncthreads();
+    }
+    if (U > 1 && u > 0) return;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      unsigned long long v = pw[q >> 1][q & 1];
+      for (int e = 1; e < U; ++e) v += sums[q * NT + e * TPU + lt];
+      if ((q & 1) == 0 || has1) atomicAdd(a.power + (long long)channel(q >> 1) * N + i0 + (q & 1), v);
     }
   }
 }

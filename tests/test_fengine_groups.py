@@ -49,3 +49,38 @@ def test_one_call_is_its_slices(N, C, T, taps, low_gain, layout):
         assert torch.equal(power, total)
         if layout == 2:
             assert int(whole[:, :, T:].count_nonzero()) == 0   # nothing past the spectra
+
+
+@pytest.mark.parametrize("N,C,T,taps", [(3, 1024, 37, 4), (2, 2048, 5, 4), (5, 64, 333, 4), (1, 256, 131, 3),
+                                        (3, 512, 70, 16), (2, 16, 1000, 1)])
+@pytest.mark.parametrize("low_gain", [False, True])
+def test_powers_of_saturating_spectra(N, C, T, taps, low_gain):
+    """Full-scale constant and alternating inputs, past the 18-bit range where
+    the transform is long enough: the power sums are those of the 18-bit
+    values, over every unit of a CTA, and add to what is there; the codes do
+    not depend on whether powers are asked for."""
+    import torch
+    from paper_1904_07778_gb300.fengine import FEngine
+    M = 2 * C
+    rng = np.random.default_rng(C + T)
+    S = (T + taps - 1) * M
+    adc = rng.integers(-20, 21, (N, S)).astype(np.int8)
+    adc[0] = 127
+    if N > 1:
+        adc[1] = np.where(np.arange(S) % 2, -127, 127)
+    gain = rng.integers(0, 140, (C, N)) if low_gain else rng.integers(120, 6000, (C, N))
+    adc = torch.from_numpy(adc).cuda()
+    with FEngine(N, C, taps) as f:
+        f.set_gains(gain.astype(np.uint32))
+        v18 = torch.empty((T, C, N, 2), dtype=torch.int32, device="cuda")
+        plain = torch.zeros((T, C, N), dtype=torch.uint8, device="cuda")
+        f.channelise(adc, T, out=plain, layout=0, v18=v18)
+        power = torch.full((C, N), 5, dtype=torch.int64, device="cuda")
+        codes = torch.zeros_like(plain)
+        f.channelise(adc, T, out=codes, layout=0, power=power)
+        f.sync()
+    v = v18.long()
+    if C >= 1024:
+        assert int(v.max()) == 131071
+    assert torch.equal(power, (v * v).sum(dim=(0, 3)) + 5)
+    assert torch.equal(codes, plain)
