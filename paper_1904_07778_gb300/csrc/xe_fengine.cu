@@ -379,11 +379,12 @@ __host__ __device__ constexpr int fe_min_blocks(int logm) { return logm <= 11 ? 
 // issue slots half busy, the shared-memory data pipe 58% and FP32 42%; the time
 // is close to proportional to the instructions of an iteration (about 1250 a
 // thread), a quarter of them the separation and equaliser.  192 inputs x 1024
-// channels x 2048 spectra: 2.02 -> 1.52 ms, in steps (ms): packed pairs and
+// channels x 2048 spectra: 2.02 -> 1.50 ms, in steps (ms): packed pairs and
 // 16-byte points 1.94; frames loaded an iteration ahead, 16 staged spectra
 // 1.78; the last pass and the separation in registers 1.59; classes within
 // warps 1.56; instances for up to four taps 1.55; the code clamped instead of
-// the spectra 1.52.
+// the spectra 1.52; no code for the other outputs, and the nibbles swapped
+// by word where real parts are low, 1.50.
 // POWER: accumulate Eq. 3's power sums, of 18-bit values clamped as integers
 // beside the equaliser's own rounding, joined over a CTA's units before they
 // are added to the caller's: ADC samples to visibilities and powers of 32 inputs
@@ -391,9 +392,13 @@ __host__ __device__ constexpr int fe_min_blocks(int logm) { return logm <= 11 ? 
 // the spectra clamped for both in floats, and every unit's sums added globally,
 // before).  FRAMED: at most four taps and
 // aligned frames, coefficients and frames in registers; otherwise any taps and
-// alignment.  (Instances of their own, so that each keeps the others'
-// registers free.)
-template <int LOGM, bool POWER, bool FRAMED>
+// alignment, the next frame's samples and coefficients read ahead (8 taps: fx
+// of 64 inputs x 512 channels x 1024 spectra 318 -> 272 us, 192 x 1024 x 2048
+// 2.54 -> 2.48 ms).  EXTRA: spectra or 18-bit values go out too (their code, in
+// the loop four times over, costs the others 2 to 4%: 192 x 256 x 4096 spectra
+// 683 -> 653 us, 192 x 1024 x 2048 1.523 -> 1.497 ms).  (Instances of their own,
+// so that each keeps the others' registers free.)
+template <int LOGM, bool POWER, bool FRAMED, bool EXTRA>
 __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine_kernel(FeArgs a) {
   constexpr int M = 1 << LOGM, C = M / 2;
   constexpr int TPU = M / 8;                 // threads per FFT unit
@@ -526,18 +531,27 @@ __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine
       }
     } else {  // any number of taps, any alignment
       uint64_t hp[4] = {0ull, 0ull, 0ull, 0ull};  // the tap before
-      for (int f = 0; f < n_act + a.taps - 1; ++f) {
-        const int8_t* xf = xt + (long long)(s + f) * M;
-        uint64_t x[2][4], hq[4] = {0ull, 0ull, 0ull, 0ull};
+      ulonglong2 hn[2];                           // the next frame's coefficients and samples
+      int2 xn[2];
+      auto load = [&](int f) {
+        hn[0] = hn[1] = make_ulonglong2(0, 0);
         if (f < a.taps) {
-          const ulonglong2 hA = __ldg(reinterpret_cast<const ulonglong2*>(a.h + f * M + 8 * lt));
-          const ulonglong2 hB = __ldg(reinterpret_cast<const ulonglong2*>(a.h + f * M + 8 * lt + 4));
-          hq[0] = hA.x, hq[1] = hA.y, hq[2] = hB.x, hq[3] = hB.y;
+          hn[0] = __ldg(reinterpret_cast<const ulonglong2*>(a.h + f * M + 8 * lt));
+          hn[1] = __ldg(reinterpret_cast<const ulonglong2*>(a.h + f * M + 8 * lt + 4));
         }
-        samples8(x[0], a.vec_in ? __ldg(reinterpret_cast<const int2*>(xf)) : load_bytes8(xf));
+        const int8_t* xf = xt + (long long)(s + f) * M;
+        xn[0] = a.vec_in ? __ldg(reinterpret_cast<const int2*>(xf)) : load_bytes8(xf);
         xf += a.adc_stride;
-        samples8(x[1], !has1 ? make_int2(0, 0)
-                             : a.vec_in ? __ldg(reinterpret_cast<const int2*>(xf)) : load_bytes8(xf));
+        xn[1] = !has1 ? make_int2(0, 0) : a.vec_in ? __ldg(reinterpret_cast<const int2*>(xf)) : load_bytes8(xf);
+      };
+      const int n_f = n_act + a.taps - 1;
+      if (n_act > 0) load(0);
+#pragma unroll 1
+      for (int f = 0; n_act > 0 && f < n_f; ++f) {
+        uint64_t x[2][4], hq[4] = {hn[0].x, hn[0].y, hn[1].x, hn[1].y};
+        samples8(x[0], xn[0]);
+        samples8(x[1], xn[1]);
+        if (f + 1 < n_f) load(f + 1);
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
           if (f < a.taps) {
@@ -591,7 +605,7 @@ __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine
         // X[input][re, im] of both spectra
         const uint64_t X[2][2] = {{p_mul(p_add(zp.x, zm.x), scale), p_mul(p_sub(zp.y, zm.y), scale)},
                                   {p_mul(p_add(zp.y, zm.y), scale), p_mul(p_sub(zm.x, zp.x), scale)}};
-        if (a.spec || a.v18) {
+        if (EXTRA && (a.spec || a.v18)) {
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
             if (j == 1 && !has1) break;
@@ -656,8 +670,9 @@ __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine
 #pragma unroll
         for (int b = 3; b >= 0; --b) {
           const int re = code_floor(q[0][b & 1][b >> 1]), im = code_floor(q[1][b & 1][b >> 1]);
-          word = a.lo_is_real ? s4_pack(im, re, word) : s4_pack(re, im, word);
+          word = s4_pack(re, im, word);
         }
+        if (a.lo_is_real) word = ((word >> 4) & 0x0F0F0F0Fu) | ((word & 0x0F0F0F0Fu) << 4);
         if (a.layout == CORR_L_CIT) {
           codes[(k * kStageIts + it % kStageIts) * NT] = word;
         } else if (a.out) {  // [t][c][i]
@@ -736,12 +751,12 @@ __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine
   }
 }
 
-template <int LOGM, bool POWER, bool FRAMED>
+template <int LOGM, bool POWER, bool FRAMED, bool EXTRA>
 cudaError_t fe_launch_one(const FeArgs& a, int n_pairs, cudaStream_t s) {
   constexpr size_t smem = fe_smem_bytes<LOGM>();
   static bool attr = false;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(fengine_kernel<LOGM, POWER, FRAMED>,
+    cudaError_t e = cudaFuncSetAttribute(fengine_kernel<LOGM, POWER, FRAMED, EXTRA>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr = true;
@@ -758,15 +773,21 @@ cudaError_t fe_launch_one(const FeArgs& a, int n_pairs, cudaStream_t s) {
   }
   const int group = b.per_unit * fe_units(LOGM);
   const dim3 grid((a.n_spectra + group - 1) / group, n_pairs);
-  fengine_kernel<LOGM, POWER, FRAMED><<<grid, fe_threads(LOGM), smem, s>>>(b);
+  fengine_kernel<LOGM, POWER, FRAMED, EXTRA><<<grid, fe_threads(LOGM), smem, s>>>(b);
   return cudaGetLastError();
 }
 
 template <int LOGM>
 cudaError_t fe_launch(const FeArgs& a, int n_pairs, cudaStream_t s) {
-  if (a.vec_in && a.taps <= 4)
-    return a.power ? fe_launch_one<LOGM, true, true>(a, n_pairs, s) : fe_launch_one<LOGM, false, true>(a, n_pairs, s);
-  return a.power ? fe_launch_one<LOGM, true, false>(a, n_pairs, s) : fe_launch_one<LOGM, false, false>(a, n_pairs, s);
+  if (a.vec_in && a.taps <= 4) {
+    if (a.spec || a.v18)
+      return a.power ? fe_launch_one<LOGM, true, true, true>(a, n_pairs, s)
+                     : fe_launch_one<LOGM, false, true, true>(a, n_pairs, s);
+    return a.power ? fe_launch_one<LOGM, true, true, false>(a, n_pairs, s)
+                   : fe_launch_one<LOGM, false, true, false>(a, n_pairs, s);
+  }
+  return a.power ? fe_launch_one<LOGM, true, false, true>(a, n_pairs, s)
+                 : fe_launch_one<LOGM, false, false, true>(a, n_pairs, s);
 }
 
 bool fe_is_device(const void* p) {
