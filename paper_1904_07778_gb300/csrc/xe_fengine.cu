@@ -761,15 +761,20 @@ cudaError_t fe_launch_one(const FeArgs& a, int n_pairs, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  // Spectra per unit: 32 (few prologues and power additions, the output's
-  // 16-spectra pieces whole), or fewer while that is less than two CTAs for
-  // every slot of the chip: 16 inputs x 128 channels x 100 spectra take 10.8 us
-  // at 2 against 18.9 us in fixed groups of 32 spectra a CTA.
+  // Spectra per unit: as many (few prologues and power additions, the output in
+  // whole pieces) as leave five CTAs for six slots of the chip: 8 inputs x 128
+  // channels x 4096 spectra 21 us at 8 (256 CTAs) against 25 and 56 at 4 and 2
+  // (a piece of two spectra leaves in bytes) and 39 at 32; 64 x 64 x 2048 33 us
+  // at 16 (256) against 39 at 4; 16 x 128 x 100 10.8 at 2 against 57 at 32.
+  // Where the output is bytes throughout, more CTAs hide more of it, two for
+  // every slot: 32 x 256 x 1000 109 us at 4 (1008 CTAs) against 117 at 16 (256).
   FeArgs b = a;
   const int slots = device_sm_count() * fe_min_blocks(LOGM);
+  const bool bytes = a.out && a.layout == CORR_L_CIT && !a.vec_out;
+  const int least = bytes ? 2 * slots : slots * 5 / 6;
   for (b.per_unit = 32; b.per_unit > 2; b.per_unit /= 2) {
     const int group = b.per_unit * fe_units(LOGM);
-    if ((long long)((a.n_spectra + group - 1) / group) * n_pairs >= 2 * slots) break;
+    if ((long long)((a.n_spectra + group - 1) / group) * n_pairs >= least) break;
   }
   const int group = b.per_unit * fe_units(LOGM);
   const dim3 grid((a.n_spectra + group - 1) / group, n_pairs);
