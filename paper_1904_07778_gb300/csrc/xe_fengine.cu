@@ -334,6 +334,28 @@ __device__ __forceinline__ uint32_t s4_pack(int hi, int lo, uint32_t low) {
   return d;
 }
 
+// n bytes of v (n = 4, 8 or 16) to any address: up to the next word by byte and
+// half word, then whole words, then the rest: 8 stores for 16 bytes instead of 16
+// (192 inputs x 1024 channels x 2047 spectra 4.1 -> 2.0 ms).  Not inlined: in
+// the kernel it costs aligned outputs 0.8%.
+__device__ __noinline__ void store_piece(uint8_t* d, uint4 v, int n) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  const int s = (int)(0u - (uint32_t)reinterpret_cast<uintptr_t>(d)) & 3;
+  if (s & 1) d[0] = (uint8_t)w[0];
+  if (s & 2) *reinterpret_cast<uint16_t*>(d + (s & 1)) = (uint16_t)(w[0] >> (8 * (s & 1)));
+  uint32_t last = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if (4 * i < n) {
+      last = __funnelshift_r(w[i], i < 3 ? w[i + 1] : 0u, 8 * s);
+      if (s == 0 || 4 * i + 4 < n) *reinterpret_cast<uint32_t*>(d + s + 4 * i) = last;
+    }
+  uint8_t* const e = d + n - 4 + s;  // 4 - s bytes remain, in `last`
+  if (s && !(s & 2)) *reinterpret_cast<uint16_t*>(e) = (uint16_t)last, last >>= 16;
+  if (s & 1) e[s & 2 ? 0 : 2] = (uint8_t)last;
+  if (s == 2) *reinterpret_cast<uint16_t*>(e) = (uint16_t)last;
+}
+
 // clamp(rne(x), -2^17, 2^17 - 1): clamping first keeps |x| < 2^22, where
 // adding 1.5 2^23 rounds x to the nearest integer, ties to even.  Returns
 // the sum's bits less those of 1.5 2^23: the integer.
@@ -700,7 +722,7 @@ __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine
           if (kk == k) nu = channel(kk);
         const uint32_t* const src = codes + k * kStageIts * NT;
         uint8_t* o = a.out + ((long long)nu * N + i0) * a.out_stride + tu + 2 * first;
-        if (a.vec_out && cnt == whole && whole >= 4) {
+        if (cnt == whole && whole >= 4) {
           uint32_t w[2][4];
 #pragma unroll
           for (int h = 0; h < 4; ++h) {
@@ -712,7 +734,9 @@ __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine
           for (int j = 0; j < 2; ++j) {
             if (j == 1 && !has1) break;
             uint8_t* d = o + j * a.out_stride;
-            if (whole == 16)
+            if (!a.vec_out)
+              store_piece(d, make_uint4(w[j][0], w[j][1], w[j][2], w[j][3]), whole);
+            else if (whole == 16)
               *reinterpret_cast<uint4*>(d) = make_uint4(w[j][0], w[j][1], w[j][2], w[j][3]);
             else if (whole == 8)
               *reinterpret_cast<uint2*>(d) = make_uint2(w[j][0], w[j][1]);
@@ -766,15 +790,16 @@ cudaError_t fe_launch_one(const FeArgs& a, int n_pairs, cudaStream_t s) {
   // channels x 4096 spectra 21 us at 8 (256 CTAs) against 25 and 56 at 4 and 2
   // (a piece of two spectra leaves in bytes) and 39 at 32; 64 x 64 x 2048 33 us
   // at 16 (256) against 39 at 4; 16 x 128 x 100 10.8 at 2 against 57 at 32.
-  // Where the output is bytes throughout, more CTAs hide more of it, two for
-  // every slot: 32 x 256 x 1000 109 us at 4 (1008 CTAs) against 117 at 16 (256).
+  // (From 32 to 16, whose pieces are as large, also where 32 leave between one
+  // and two CTAs a slot: 32 x 256 x 4096 with powers, to visibilities, 174 us at
+  // 16 against 180 at 32, 512 CTAs.)
   FeArgs b = a;
   const int slots = device_sm_count() * fe_min_blocks(LOGM);
-  const bool bytes = a.out && a.layout == CORR_L_CIT && !a.vec_out;
-  const int least = bytes ? 2 * slots : slots * 5 / 6;
   for (b.per_unit = 32; b.per_unit > 2; b.per_unit /= 2) {
     const int group = b.per_unit * fe_units(LOGM);
-    if ((long long)((a.n_spectra + group - 1) / group) * n_pairs >= least) break;
+    const long long ctas = (long long)((a.n_spectra + group - 1) / group) * n_pairs;
+    if (b.per_unit == 32 && ctas > slots && ctas < 2 * slots) continue;
+    if (ctas >= slots * 5 / 6) break;
   }
   const int group = b.per_unit * fe_units(LOGM);
   const dim3 grid((a.n_spectra + group - 1) / group, n_pairs);

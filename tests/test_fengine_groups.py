@@ -84,3 +84,29 @@ def test_powers_of_saturating_spectra(N, C, T, taps, low_gain):
         assert int(v.max()) == 131071
     assert torch.equal(power, (v * v).sum(dim=(0, 3)) + 5)
     assert torch.equal(codes, plain)
+
+
+@pytest.mark.parametrize("N,C,T", [(3, 64, 2), (2, 64, 7), (5, 128, 67), (4, 64, 1030), (7, 1024, 45), (2, 2048, 19),
+                                   (16, 64, 4099)])
+@pytest.mark.parametrize("shift,pad", [(1, 0), (2, 3), (3, 1), (0, 5), (8, 4)])
+def test_codes_to_any_address(N, C, T, shift, pad):
+    """Rows of codes at any address and stride equal those of aligned rows,
+    and nothing is written between them."""
+    import torch
+    from paper_1904_07778_gb300.fengine import FEngine
+    taps, M = 4, 2 * C
+    g = torch.Generator(device="cuda").manual_seed(N * C + T)
+    adc = torch.randint(-100, 101, (N, (T + taps - 1) * M), generator=g, device="cuda", dtype=torch.int8)
+    gain = np.random.default_rng(T).integers(100, 3000, (C, N)).astype(np.uint32)
+    stride = (T + 15) // 16 * 16
+    with FEngine(N, C, taps) as f:
+        f.set_gains(gain)
+        want = torch.zeros((C, N, stride), dtype=torch.uint8, device="cuda")
+        f.channelise(adc, T, out=want, layout=2, out_stride=stride)
+        buf = torch.full((shift + C * N * (T + pad) + 16,), 0x5A, dtype=torch.uint8, device="cuda")
+        f.channelise(adc, T, out=buf[shift:], layout=2, out_stride=T + pad)
+        f.sync()
+    rows = buf[shift:shift + C * N * (T + pad)].view(C, N, T + pad)
+    assert torch.equal(rows[:, :, :T], want[:, :, :T])
+    assert bool((rows[:, :, T:] == 0x5A).all())
+    assert bool((buf[:shift] == 0x5A).all()) and bool((buf[shift + C * N * (T + pad):] == 0x5A).all())
