@@ -45,6 +45,7 @@ struct FeArgs {
   float* spec;
   unsigned long long* power;
   int n_inputs, n_spectra, taps, layout;
+  int pairs_first;  // CTAs in order of input pairs, not of groups of spectra
   int per_unit;  // consecutive spectra of each FFT unit: 2, 4, 8, 16 or 32
   int lo_is_real, vec_in, vec_out;
   float scale;  // 2^-(shift + 1): Eq. 2's halving and the 18-bit scaling
@@ -438,13 +439,16 @@ __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine
   // their clamp bounds, bfloat16 each (registers are what limits the CTA)
   float2* const gains = reinterpret_cast<float2*>(codes - tid + 4 * kStageIts * NT) + tid;
   uint32_t* const bounds = reinterpret_cast<uint32_t*>(gains - tid + 4 * NT) + tid;
-  const int i0 = 2 * blockIdx.y;
+  const int i0 = 2 * (a.pairs_first ? blockIdx.x : blockIdx.y);
+  const int grp = a.pairs_first ? blockIdx.y : blockIdx.x;  // the CTA's group of spectra
   const bool has1 = i0 + 1 < a.n_inputs;
   const int N = a.n_inputs;
+  // [t][c][i] codes: both inputs' as one half word
+  const bool pair16 = has1 && ((N | (int)reinterpret_cast<uintptr_t>(a.out)) & 1) == 0;
   // this unit's spectra tu .. tu + per_unit - 1, two an iteration; the first
   // unit's range, the earliest, says how many iterations the CTA makes
-  const int tu = (blockIdx.x * U + u) * a.per_unit;
-  const int n_it = (min(a.per_unit, a.n_spectra - (int)blockIdx.x * U * a.per_unit) + 1) / 2;
+  const int tu = (grp * U + u) * a.per_unit;
+  const int n_it = (min(a.per_unit, a.n_spectra - grp * U * a.per_unit) + 1) / 2;
 
   // per-thread constants: the filter taps of its 8 samples (neighbouring
   // samples in pairs; absent taps are zeros) and the twiddles of every pass
@@ -702,6 +706,10 @@ __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
             if (e >= n_act) break;
+            if (pair16) {
+              *reinterpret_cast<uint16_t*>(o + (long long)e * C * N) = (uint16_t)(word >> (16 * e));
+              continue;
+            }
             o[(long long)e * C * N] = (uint8_t)(word >> (16 * e));
             if (has1) o[(long long)e * C * N + 1] = (uint8_t)(word >> (16 * e + 8));
           }
@@ -802,7 +810,13 @@ cudaError_t fe_launch_one(const FeArgs& a, int n_pairs, cudaStream_t s) {
     if (ctas >= slots * 5 / 6) break;
   }
   const int group = b.per_unit * fe_units(LOGM);
-  const dim3 grid((a.n_spectra + group - 1) / group, n_pairs);
+  // [t][c][i] codes: CTAs of neighbouring pairs, which write the same sectors, run
+  // together, so that the L2 joins their bytes (192 inputs x 1024 channels x 2048
+  // spectra 5.5 -> 2.35 ms; the half-word stores alone 5.1, and 64 x 512 x 2048
+  // 480 -> 315 us).
+  const int groups = (a.n_spectra + group - 1) / group;
+  b.pairs_first = a.out && a.layout != CORR_L_CIT && groups <= 65535;
+  const dim3 grid = b.pairs_first ? dim3(n_pairs, groups) : dim3(groups, n_pairs);
   fengine_kernel<LOGM, POWER, FRAMED, EXTRA><<<grid, fe_threads(LOGM), smem, s>>>(b);
   return cudaGetLastError();
 }
