@@ -110,3 +110,30 @@ def test_codes_to_any_address(N, C, T, shift, pad):
     assert torch.equal(rows[:, :, :T], want[:, :, :T])
     assert bool((rows[:, :, T:] == 0x5A).all())
     assert bool((buf[:shift] == 0x5A).all()) and bool((buf[shift + C * N * (T + pad):] == 0x5A).all())
+
+
+@pytest.mark.parametrize("N,C,T,taps", [(2, 64, 5, 4), (3, 64, 37, 4), (6, 256, 33, 3), (5, 1024, 9, 4), (4, 128, 21, 6)])
+@pytest.mark.parametrize("shift", [0, 2])
+def test_spectra_and_values_at_any_alignment(N, C, T, taps, shift):
+    """The FP32 spectra and 18-bit values, alone and together, at 16- and
+    8-byte aligned addresses: the values are the spectra rounded and clamped,
+    and the same every way."""
+    import torch
+    from paper_1904_07778_gb300.fengine import FEngine
+    M, n = 2 * C, T * C * N * 2
+    g = torch.Generator(device="cuda").manual_seed(N * C + T)
+    adc = torch.randint(-127, 128, (N, (T + taps - 1) * M), generator=g, device="cuda", dtype=torch.int8)
+    adc[0] = 127
+    sp = torch.full((2, n + 8), 7.0, device="cuda")
+    v18 = torch.full((2, n + 8), 7, dtype=torch.int32, device="cuda")
+    with FEngine(N, C, taps) as f:
+        f.set_gains(np.full((C, N), 900, np.uint32))
+        f.channelise(adc, T, spec=sp[0, shift:], v18=v18[0, shift:])
+        f.channelise(adc, T, spec=sp[1, 4:])
+        f.channelise(adc, T, v18=v18[1, 4:])
+        f.sync()
+    a, v = sp[0, shift:shift + n], v18[0, shift:shift + n]
+    assert torch.equal(a, sp[1, 4:4 + n]) and torch.equal(v, v18[1, 4:4 + n])
+    assert torch.equal(v, a.double().round().clamp(-131072, 131071).int())
+    for buf, s in ((sp[0], shift), (v18[0], shift), (sp[1], 4), (v18[1], 4)):
+        assert bool((buf[:s] == 7).all()) and bool((buf[s + n:] == 7).all())
