@@ -1141,7 +1141,16 @@ __global__ void __launch_bounds__(kRingThreads, 1)
 #undef budget
   tc_before_sync();
   __syncthreads();
-  if (PAIR) cluster_sync();  // neither CTA's shared or tensor memory is in use by the other's work
+  if (PAIR) {
+    // CTA 0's commits arrive on CTA 1's barriers too: the last of them, `done`,
+    // which follows every MMA, has to be here before CTA 1 leaves and its shared
+    // memory is another's.  (CTA 0 always commits it, at the latest when its own
+    // waits have run out.)
+    int never = 0;
+    if (rank == 1 && warp == kMmaWarp && lane == 0 && !mbar_wait(&sm.done, 0, &never)) raise_timeout(a, abort);
+    __syncwarp();
+    cluster_sync();  // neither CTA's shared or tensor memory is in use by the other's work
+  }
   if (warp == 0) {
     if (PAIR)
       tmem_free_pair(tmem, 512);
