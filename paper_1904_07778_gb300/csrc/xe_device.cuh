@@ -25,38 +25,54 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(smem_addr(bar))
                : "memory");
 }
+// CLUSTER: the wait acquires what arrivals of the cluster's other CTA released
+// (the default scope, the CTA, leaves those out).
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
-  asm volatile(
-      "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      "selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(smem_addr(bar)), "r"(parity)
-      : "memory");
+  if constexpr (CLUSTER)
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
+  else
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
   return ok != 0;
 }
 // Wait until the phase with the given parity has completed, or give up when
 // *abort is set or after 2^budget_log2 cycles (default kWaitCycles).
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
                                           int budget_log2 = 31) {
-  if (mbar_test(bar, parity)) return true;
+  if (mbar_test<CLUSTER>(bar, parity)) return true;
   const long long t0 = clock64();
-  while (!mbar_test(bar, parity)) {
+  while (!mbar_test<CLUSTER>(bar, parity)) {
     if (*abort) return false;
     if ((clock64() - t0) >> budget_log2) return false;
   }
   return true;
 }
 
-// Arrive on the barrier at the same place in CTA `rank` of the cluster.  (What
-// the arrival announces is operands and accumulators of this thread's own SM,
-// which the proxy fence and the tcgen05 fence before it have completed there;
-// a release over the cluster on top cost the pair's unpack a third of its
-// time.)
+// Arrive on the barrier at the same place in CTA `rank` of the cluster, after
+// this CTA's shared memory has been released over the cluster: operands that
+// this warp has written, for MMAs that a thread of CTA `rank` issues once its
+// mbar_wait<true> has acquired them.  (An arrival without qualifiers releases at
+// CTA scope only, which promises nothing to that thread.  The fence is kept to
+// shared memory: with a release of everything, mbarrier.arrive.release.cluster,
+// 512 inputs x 304 channels x 4096 spectra take 1.45 ms, or 2.05 with one
+// thread passing on a CTA's stages; 1.13 with this fence, as without one.)
 __device__ __forceinline__ void mbar_arrive_cluster(uint64_t* bar, uint32_t rank) {
   asm volatile(
       "{\n.reg .b32 ra;\nmapa.shared::cluster.u32 ra, %0, %1;\n"
-      "mbarrier.arrive.shared::cluster.b64 _, [ra];\n}\n" ::"r"(smem_addr(bar)),
+      "fence.release.sync_restrict::shared::cta.cluster;\n"
+      "mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [ra];\n}\n" ::"r"(smem_addr(bar)),
       "r"(rank)
       : "memory");
 }

@@ -822,7 +822,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
           const int b = v & 1;
           const int k0 = EIGHT ? q * piece_stages<EIGHT>(g.dbl) : 0;
           const int k1 = EIGHT ? min(nk, k0 + piece_stages<EIGHT>(g.dbl)) : nk;
-          if (v >= 2 && !mbar_wait(&sm.tmem_empty[b], (uint32_t)(((v >> 1) - 1) & 1), abort, budget)) {
+          if (v >= 2 && !mbar_wait<PAIR>(&sm.tmem_empty[b], (uint32_t)(((v >> 1) - 1) & 1), abort, budget)) {
             raise_timeout(a, abort);
             ok = false;
             break;
@@ -833,7 +833,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
           auto issue = [&](auto DBL) {
             constexpr bool dbl = decltype(DBL)::value;
             for (int k = k0; k < k1; ++k) {
-              if (!mbar_wait(&sm.full_o[s], (uint32_t)(m & 1), abort, budget)) {
+              if (!mbar_wait<PAIR>(&sm.full_o[s], (uint32_t)(m & 1), abort, budget)) {
                 raise_timeout(a, abort);
                 ok = false;
                 break;

@@ -30,3 +30,26 @@ def test_pairs_of_one_stage_leave_one_after_the_other(N, C, T):
             cor.push(d)
         vis = cor.dump()
     assert np.array_equal(vis, n * oracle.correlate(b, N, C, T, bits=8, layout=xe.CORR_L_CIT))
+
+
+@pytest.mark.parametrize("N,C,T,layout", [(512, 4, 4100, 0), (320, 40, 2048, 2)])
+def test_long_runs_of_pairs_repeat(N, C, T, layout):
+    """Thousands of stages whose operands one CTA of a pair writes and the
+    other's MMAs read, accumulators reused every 1024 spectra: every
+    integration of one block equals the first, and that the oracle's."""
+    import torch
+    from paper_1904_07778_gb300 import xengine as xe
+    b = _block(N + T, 2 * N * C * T)
+    d = torch.from_numpy(b).cuda()
+    with xe.Correlator(N, C, T, bits=8, layout=layout) as cor:
+        vis = torch.empty((2, C, N * (N + 1) // 2, 2), dtype=torch.int64, device="cuda")
+        cor.push(d)
+        cor.dump_into(vis[0])
+        for _ in range(60):
+            cor.push(d)
+            cor.dump_into(vis[1])
+            assert torch.equal(vis[0], vis[1])
+    c = 1 if N == 512 else C // 2   # the oracle: one channel
+    x = b.reshape((T, C, N, 2) if layout == 0 else (C, N, T, 2))
+    one = np.ascontiguousarray(x[:, c] if layout == 0 else x[c])
+    assert np.array_equal(vis[0][c:c + 1].cpu().numpy(), oracle.correlate(one, N, 1, T, bits=8, layout=layout))
