@@ -304,8 +304,9 @@ typedef struct corr_stats {
  *                 instead of the default budget of 2^31 (about a second);
  *                 0 restores the default.
  * The visibilities of a push made with a fault are undefined and its dump
- * returns CORR_ETIMEDOUT.  Only the 4-bit TMA path of corr_push (row
- * strides that are multiples of 16 bytes) reads the hook.  Waits for the
+ * returns CORR_ETIMEDOUT.  Only the TMA path of corr_push (4-bit row
+ * strides that are multiples of 16 bytes, and every 8-bit block, whose stages
+ * are 64 spectra) reads the hook.  Waits for the
  * context's work first.  CORR_EINVAL for stage outside -1 .. 2^24 - 2 or
  * wait_log2 outside 0 .. 40.
  */

@@ -11,7 +11,6 @@ namespace xe {
 
 // Cycle budget of one bounded wait (about a second at GB300 clocks).
 constexpr long long kWaitCycles = 1ll << 31;
-static_assert(kWaitCycles == (1ll << 31), "mbar_wait's default budget_log2 is 31");
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -47,15 +46,15 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 // Wait until the phase with the given parity has completed, or give up when
-// *abort is set or after 2^budget_log2 cycles (default kWaitCycles).
+// *abort is set or after `budget` cycles.
 template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
-                                          int budget_log2 = 31) {
+                                          long long budget = kWaitCycles) {
   if (mbar_test<CLUSTER>(bar, parity)) return true;
   const long long t0 = clock64();
   while (!mbar_test<CLUSTER>(bar, parity)) {
     if (*abort) return false;
-    if ((clock64() - t0) >> budget_log2) return false;
+    if (clock64() - t0 >= budget) return false;
   }
   return true;
 }

@@ -698,9 +698,8 @@ __global__ void __launch_bounds__(kRingThreads, 1)
     return;
   }
   volatile int* abort = &sm.abort;
-  // every wait's budget, log2 cycles: w if the fault field sets it (only the
-  // fault-injection tests shorten it), read from the parameter space at each wait
-#define budget ((!EIGHT && (a.in.fault >> 24)) ? (a.in.fault >> 24) : 31)
+  // every wait's budget in cycles, read from the parameter space at each
+#define budget a.wait_cycles
 
   // The loader sets up the barriers and does not wait for the other warps'
   // part (row sums, tensor memory): its first loads are on their way while
@@ -1380,6 +1379,7 @@ cudaError_t herk4_launch(const HerkArgs& args, const CUtensorMap* tmap, int n_ta
   if (tmap || args.tmaps) {
     HerkArgs a = args;
     a.smem_bytes = ring_smem();
+    a.wait_cycles = a.in.fault >> 24 ? 1ll << (a.in.fault >> 24) : kWaitCycles;
     // four slots, the control block and the alignment pad
     if (a.smem_bytes < kGroups * kSlotBytes + (int)sizeof(RingCtrl) + 1024)
       return cudaErrorInvalidConfiguration;

@@ -89,6 +89,7 @@ struct HerkArgs {
   int2* scratch;
   int scratch_ctas;
   int smem_bytes;            // dynamic shared memory of the launch
+  long long wait_cycles;     // limit of every wait: set by herk4_launch from in.fault
   int n_tasks;               // tasks in `tasks`
   int grid;                  // CTAs of a launch with cta_first; otherwise, if > 0,
                              // the most CTAs (SMs) a single-array launch may use
