@@ -302,7 +302,8 @@ typedef struct corr_stats {
  *                 list), so the waits for it run out; -1 turns it off.
  *   wait_log2   : 1 .. 40 limits every wait to 2^wait_log2 SM cycles
  *                 instead of the default budget of 2^31 (about a second);
- *                 0 restores the default.
+ *                 0 restores the default.  (The last waits, for the copies
+ *                 and MMAs in flight when a role leaves, keep the default.)
  * The visibilities of a push made with a fault are undefined and its dump
  * returns CORR_ETIMEDOUT.  Only the TMA path of corr_push (4-bit row
  * strides that are multiples of 16 bytes, and every 8-bit block, whose stages

@@ -799,10 +799,11 @@ __global__ void __launch_bounds__(kRingThreads, 1)
           ++m;
         }
       }
-      // never leave with copies in flight: wait for the last loads to land
+      // never leave with copies in flight: wait for the last loads to land (they
+      // do, whatever gave up, so a shortened limit is not for these waits)
       int never = 0;
       for (int S = issued - 1; S >= 0 && S >= issued - ns; --S)
-        if (S != skip) mbar_wait(&sm.full_t[S % ns], (uint32_t)((S / ns) & 1), &never, budget);
+        if (S != skip) mbar_wait(&sm.full_t[S % ns], (uint32_t)((S / ns) & 1), &never);
     }
     __syncwarp();
   } else if (warp == kMmaWarp) {
@@ -881,8 +882,8 @@ __global__ void __launch_bounds__(kRingThreads, 1)
         umma_commit_pair(&sm.done);
       else
         umma_commit(&sm.done);
-      int never = 0;
-      if (!mbar_wait(&sm.done, 0, &never, budget)) raise_timeout(a, abort);
+      int never = 0;  // the MMAs in flight end: the default limit, as for the loads
+      if (!mbar_wait(&sm.done, 0, &never)) raise_timeout(a, abort);
     }
     __syncwarp();
   } else if (warp < kUnpackWarps) {

@@ -46,3 +46,26 @@ def test_withheld_stage_at_8_bits(N, C, T, stage, layout):
     x = blocks[1].reshape((T, C, N, 2) if layout == 0 else (C, N, T, 2))
     one = np.ascontiguousarray(x[:, c] if layout == 0 else x[c])
     assert np.array_equal(vis[c:], oracle.correlate(one, N, 1, T, bits=8, layout=layout))
+
+
+@pytest.mark.parametrize("N,C,T,bits", [(32, 64, 1024, 4), (192, 8, 2048, 4), (192, 4, 1024, 8), (256, 8, 1024, 8)])
+@pytest.mark.parametrize("wait_log2", [1, 9, 12])
+def test_limits_shorter_than_a_load(N, C, T, bits, wait_log2):
+    """Limits that run out while loads and MMAs are in flight: the roles give
+    up, what is in flight still lands before the CTA leaves, and the next
+    integration is exact."""
+    from paper_1904_07778_gb300 import xengine as xe
+    b = synth.random_bytes(5 + N, N * C * T * bits // 4)
+    b[b == 0x80] = 0x81
+    dev = torch.from_numpy(b).cuda()
+    want = oracle.correlate(b, N, C, T, bits=bits, layout=2)
+    with xe.Correlator(N, C, T, bits=bits, layout=2) as cor:
+        for _ in range(20):
+            cor.set_fault_injection(-1, wait_log2=wait_log2)
+            cor.push(dev)
+            vis = cor.dump(check=False)
+            assert cor.last_status in (xe.CORR_OK, xe.CORR_ETIMEDOUT)
+            assert cor.last_status == xe.CORR_ETIMEDOUT or np.array_equal(vis, want)
+            cor.set_fault_injection(-1, 0)
+            cor.push(dev)
+            assert np.array_equal(cor.dump(), want)
