@@ -449,6 +449,10 @@ int64_t* corr_batch_output(corr_batch* b, int k);
 int corr_batch_set_input(corr_batch* b, int k, const void* src, size_t nbytes);
 int corr_batch_get_output(corr_batch* b, int k, int64_t* dst);
 
+/* The cudaStream_t of the batch's copies and runs (its private one, or the
+ * caller's), for ordering other work with them.  NULL for a null batch. */
+void* corr_batch_stream(corr_batch* b);
+
 /* corr_batch_run -- correlate the current block of every array (the outputs
  * are overwritten, not accumulated): replays the batch's CUDA graph on its
  * stream.  Asynchronous. */

@@ -497,6 +497,8 @@ int64_t* corr_batch_output(corr_batch* b, int k) {
   return (b && k >= 0 && k < b->n) ? b->acc[k] : nullptr;
 }
 
+void* corr_batch_stream(corr_batch* b) { return b ? (void*)b->stream : nullptr; }
+
 int corr_batch_set_input(corr_batch* b, int k, const void* src, size_t nbytes) {
   if (!b || k < 0 || k >= b->n || !src) return CORR_EINVAL;
   const corr_shape& s = b->shapes[k];

@@ -10,6 +10,7 @@ tensors (host or device).
 """
 from __future__ import annotations
 
+import collections
 import ctypes
 import os
 
@@ -180,6 +181,42 @@ def _ptr_and_size(buf):
             raise ValueError("tensor must be contiguous")
         return buf.data_ptr(), buf.numel() * buf.element_size()
     raise TypeError("expected a numpy array or a torch tensor")
+
+
+class _CopyStream:
+    """Copies out of torch tensors on a stream of the library's: each waits for
+    what torch's current stream has queued (the tensor's producer, usually),
+    and the tensor lives until its copy is done."""
+
+    def __init__(self, handle):
+        self._handle, self._stream, self._busy = handle, None, collections.deque()
+
+    def before(self, src):
+        if not getattr(src, "is_cuda", False):
+            return
+        import torch
+        if self._stream is None:
+            self._stream = torch.cuda.ExternalStream(self._handle)
+        cur = torch.cuda.current_stream()
+        if cur.cuda_stream != self._handle and not torch.cuda.is_current_stream_capturing():
+            self._stream.wait_stream(cur)
+
+    def after(self, src):
+        if not hasattr(src, "data_ptr"):
+            return
+        import torch
+        if not torch.cuda.is_available():
+            return
+        if self._stream is None:
+            self._stream = torch.cuda.ExternalStream(self._handle)
+        while self._busy and self._busy[0][0].query():
+            self._busy.popleft()
+        done = torch.cuda.Event()
+        done.record(self._stream)
+        self._busy.append((done, src))
+
+    def synchronised(self):
+        self._busy.clear()
 
 
 class Correlator:
@@ -357,7 +394,8 @@ class Correlator:
 # ------------------------------------------------------------------- batches
 EXPORTS += ["corr_batch_create", "corr_batch_input", "corr_batch_output", "corr_batch_set_input",
             "corr_batch_get_output", "corr_batch_run", "corr_batch_run_plain", "corr_batch_sync",
-            "corr_batch_info_get", "corr_batch_destroy", "corr_plan_schedule", "corr_batch_set_pipeline"]
+            "corr_batch_info_get", "corr_batch_destroy", "corr_plan_schedule", "corr_batch_set_pipeline",
+            "corr_batch_stream"]
 CORR_SCHED_PAIRS_LPT, CORR_SCHED_SINGLES_LPT, CORR_SCHED_PAIRS_RR = 0, 1, 2
 
 
@@ -380,6 +418,8 @@ _lib.corr_batch_output.argtypes = [_P, _I]
 _lib.corr_batch_output.restype = _P
 _lib.corr_batch_set_input.argtypes = [_P, _I, _P, _SZ]
 _lib.corr_batch_get_output.argtypes = [_P, _I, _P]
+_lib.corr_batch_stream.argtypes = [_P]
+_lib.corr_batch_stream.restype = _P
 _lib.corr_batch_run.argtypes = [_P]
 _lib.corr_batch_run_plain.argtypes = [_P]
 _lib.corr_batch_set_pipeline.argtypes = [_P, _I, _I]
@@ -426,12 +466,19 @@ class Batch:
         if st != CORR_OK:
             raise CorrError(st, "corr_batch_create")
         self._b = out
+        self._copies = _CopyStream(_lib.corr_batch_stream(out))
 
     def set_input(self, k, block):
+        """Queue the copy of ``block`` (host or device) into array k's input.
+        A torch tensor's copy follows the work queued on torch's current
+        stream, and the tensor is kept until it is done; its contents may be
+        changed after :meth:`sync`."""
         p, n = _ptr_and_size(block)
+        self._copies.before(block)
         st = _lib.corr_batch_set_input(self._b, k, _P(p), n)
         if st != CORR_OK:
             raise CorrError(st, "corr_batch_set_input")
+        self._copies.after(block)
 
     def output(self, k):
         n, c = self.shapes[k][0], self.shapes[k][1]
@@ -439,6 +486,7 @@ class Batch:
         st = _lib.corr_batch_get_output(self._b, k, _P(vis.ctypes.data))
         if st != CORR_OK:
             raise CorrError(st, "corr_batch_get_output")
+        self._copies.synchronised()
         return vis
 
     def run(self):
@@ -460,7 +508,9 @@ class Batch:
             raise CorrError(st, "corr_batch_set_pipeline")
 
     def sync(self):
-        return _lib.corr_batch_sync(self._b)
+        st = _lib.corr_batch_sync(self._b)
+        self._copies.synchronised()
+        return st
 
     def info(self):
         out = CorrBatchInfo()
@@ -475,6 +525,7 @@ class Batch:
         if getattr(self, "_b", None):
             _lib.corr_batch_destroy(self._b)
             self._b = None
+            self._copies.synchronised()
 
     def __enter__(self):
         return self
