@@ -93,7 +93,10 @@ typedef struct corr_ctx corr_ctx; /* opaque, owned by the library */
  *   stream   : cudaStream_t to run on, or NULL for a private stream.
  *   out      : receives the context.
  * Allocates the context's device state (accumulators, staging, corner-turn
- * buffers) on the current device.  Returns CORR_EINVAL for a bad shape,
+ * buffers; for 4-bit CORR_L_CIT with T not a multiple of 16 also rows padded
+ * for faster reads, where they take at most an eighth of the free memory and
+ * until another allocation of the context needs their room) on the current
+ * device.  Returns CORR_EINVAL for a bad shape,
  * CORR_ENOMEM when an allocation fails, CORR_ECUDA when no usable device.
  */
 int corr_create(int n_inputs, int n_chans, int n_time, int bits, int layout, unsigned flags,

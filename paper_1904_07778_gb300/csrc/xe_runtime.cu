@@ -172,6 +172,7 @@ struct corr_ctx {
   cudaEvent_t stage_ready[2] = {nullptr, nullptr};
   int stage_next = 0;
   uint8_t* turned = nullptr;  // corner-turned copy of the block, [c][i][t] (= turned_buf[0])
+  bool spare_turned = false;  // `turned` holds padded rows, which the context can do without
   // Pipelined corner turn (corr_set_pipeline): the turn of block k+1 runs on
   // pipe_sms SMs of turn_stream while the cross-multiply of block k holds the
   // other SMs on herk_stream; the two turned buffers alternate.
@@ -319,6 +320,26 @@ bool is_device_ptr(const void* p) {
     return false;
   }
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
+}
+
+// Device memory of a context that is running.  Short of memory, it gives up
+// its padded rows (pushes then read the blocks' own rows, slower), so that it
+// needs no more than it would without them; not once a push was captured,
+// whose graph has their address.  (The error is the call's, not the thread's
+// last one, which the caller's own checks would take for theirs.)
+cudaError_t ctx_alloc(corr_ctx* x, void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) cudaGetLastError();
+  if (e != cudaErrorMemoryAllocation || !x->spare_turned) return e;
+  if ((e = cudaStreamSynchronize(x->stream)) != cudaSuccess) return e;
+  for (auto& c : x->map_cache)
+    if (c.src == x->turned) c.src = nullptr;
+  if ((e = cudaFree(x->turned)) != cudaSuccess) return e;
+  x->turned = x->turned_buf[0] = nullptr;
+  x->spare_turned = false;
+  e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
 }
 
 void free_ctx(corr_ctx* x) {
@@ -506,12 +527,19 @@ int corr_create(int n_inputs, int n_chans, int n_time, int bits, int layout, uns
     // by TMA: a push copies them to padded rows first (pad_rows_launch).  That
     // is one more pass over the block, but the kernel that loads any row
     // without TMA is several times slower (192 inputs x 256 channels x 4097
-    // spectra: 0.18 against 1.75 ms a push and dump).  Without memory for
-    // the copy that kernel still serves.
-    if (layout == CORR_L_CIT && bits == 4 && n_time % 16 != 0 &&
-        cudaMalloc(&x->turned, (size_t)x->turned_stride * byte_rows * n_chans) != cudaSuccess) {
-      cudaGetLastError();
-      x->turned = nullptr;
+    // spectra: 0.18 against 1.75 ms a push and dump).  Where the copy would
+    // take more than an eighth of the free memory, or nothing is left for it,
+    // that kernel still serves, and it does again once an allocation of the
+    // context needs the memory (ctx_alloc).
+    if (layout == CORR_L_CIT && bits == 4 && n_time % 16 != 0) {
+      const size_t bytes = (size_t)x->turned_stride * byte_rows * n_chans;
+      size_t free_bytes = 0, total = 0;
+      if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess || bytes > free_bytes / 8 ||
+          cudaMalloc(&x->turned, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        x->turned = nullptr;
+      }
+      x->spare_turned = x->turned != nullptr;
     }
     x->turned_buf[0] = x->turned;
     if (cudaMalloc(&x->d_status, sizeof(int)) != cudaSuccess) { st = CORR_ENOMEM; break; }
@@ -585,7 +613,7 @@ int corr_push(corr_ctx* x, const void* block, size_t nbytes, uint64_t seq) {
   if (!on_device) {
     slot = x->stage_next;
     x->stage_next ^= 1;
-    if (!x->stage[slot] && cudaMalloc(&x->stage[slot], x->block_bytes) != cudaSuccess)
+    if (!x->stage[slot] && ctx_alloc(x, (void**)&x->stage[slot], x->block_bytes) != cudaSuccess)
       return CORR_ENOMEM;
     if (cudaStreamWaitEvent(x->copy_stream, x->stage_free[slot], 0) != cudaSuccess)
       return CORR_ECUDA;
@@ -618,6 +646,10 @@ int corr_push(corr_ctx* x, const void* block, size_t nbytes, uint64_t seq) {
     src = turned;
     row_stride = x->turned_stride;
   } else if (!needs_turn(x->layout, x->bits) && T % 16 != 0 && x->turned) {
+    cudaStreamCaptureStatus captured = cudaStreamCaptureStatusNone;
+    if (x->spare_turned && cudaStreamIsCapturing(ts, &captured) == cudaSuccess &&
+        captured != cudaStreamCaptureStatusNone)
+      x->spare_turned = false;  // a graph will keep the address
     cudaEvent_t tt = phase_begin(x, ts);
     cudaError_t e = pad_rows_launch(src, x->turned, (long long)R * C, T, x->turned_stride, ts);
     if (e != cudaSuccess) return cuda_fail(e);
@@ -933,7 +965,7 @@ int corr_dump_async(corr_ctx* x, int64_t* vis, int reset) {
       return CORR_ECUDA;
     }
   }
-  if (reset && !x->acc_buf[1] && cudaMalloc(&x->acc_buf[1], x->acc_bytes) != cudaSuccess)
+  if (reset && !x->acc_buf[1] && ctx_alloc(x, (void**)&x->acc_buf[1], x->acc_bytes) != cudaSuccess)
     return CORR_ENOMEM;
   if (!x->acc_live) {  // nothing pushed since the last reset: an all-zero integration
     if (int g = guard_acc_write(x, as)) return g;
@@ -1076,13 +1108,13 @@ int corr_normalise_flags(corr_ctx* x, double* rho, uint8_t* zero_flag) {
   const bool dev = is_device_ptr(rho);
   double* d = rho;
   if (!dev) {
-    if (!x->rho_tmp && cudaMalloc(&x->rho_tmp, bytes) != cudaSuccess) return CORR_ENOMEM;
+    if (!x->rho_tmp && ctx_alloc(x, (void**)&x->rho_tmp, bytes) != cudaSuccess) return CORR_ENOMEM;
     d = x->rho_tmp;
   }
   const bool fdev = zero_flag && is_device_ptr(zero_flag);
   uint8_t* f = zero_flag;
   if (zero_flag && !fdev) {
-    if (!x->flag_tmp && cudaMalloc(&x->flag_tmp, flag_bytes) != cudaSuccess) return CORR_ENOMEM;
+    if (!x->flag_tmp && ctx_alloc(x, (void**)&x->flag_tmp, flag_bytes) != cudaSuccess) return CORR_ENOMEM;
     f = x->flag_tmp;
   }
   cudaEvent_t tn = phase_begin(x, x->stream);
