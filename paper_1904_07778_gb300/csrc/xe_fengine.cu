@@ -48,6 +48,7 @@ struct FeArgs {
   int pairs_first;  // CTAs in order of input pairs, not of groups of spectra
   int per_unit;  // consecutive spectra of each FFT unit: 2, 4, 8, 16 or 32
   int lo_is_real, vec_in, vec_out;
+  int vec_two;  // [c][i][t] pieces of two spectra leave as half words
   int vec_extra;  // both inputs' spectra and 18-bit values as 16 bytes
   float scale;  // 2^-(shift + 1): Eq. 2's halving and the 18-bit scaling
 };
@@ -767,6 +768,10 @@ __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine
             else
               *reinterpret_cast<uint32_t*>(d) = w[j][0];
           }
+        } else if (a.vec_two && cnt == 2) {
+          const uint32_t w = src[0];
+          *reinterpret_cast<uint16_t*>(o) = (uint16_t)__byte_perm(w, 0u, 0x4420);
+          if (has1) *reinterpret_cast<uint16_t*>(o + a.out_stride) = (uint16_t)__byte_perm(w, 0u, 0x4431);
         } else {
           for (int q = 0; q < cnt; ++q) {
             const uint32_t w = src[(q >> 1) * NT] >> (16 * (q & 1));
@@ -811,20 +816,30 @@ cudaError_t fe_launch_one(const FeArgs& a, int n_pairs, cudaStream_t s) {
   }
   // Spectra per unit: as many (few prologues and power additions, the output in
   // whole pieces) as leave five CTAs for six slots of the chip: 8 inputs x 128
-  // channels x 4096 spectra 21 us at 8 (256 CTAs) against 25 and 56 at 4 and 2
-  // (a piece of two spectra leaves in bytes) and 39 at 32; 64 x 64 x 2048 33 us
-  // at 16 (256) against 39 at 4; 16 x 128 x 100 10.8 at 2 against 57 at 32.
+  // channels x 4096 spectra 21 us at 8 (256 CTAs) against 25 at 4 and 39 at 32;
+  // 64 x 64 x 2048 33 us at 16 (256) against 39 at 4; 16 x 128 x 100 10.8 at 2
+  // against 57 at 32.
   // (From 32 to 16, whose pieces are as large, also where 32 leave between one
   // and two CTAs a slot: 32 x 256 x 4096 with powers, to visibilities, 174 us at
   // 16 against 180 at 32, 512 CTAs.)
+  // Where the pieces of [c][i][t] codes are whole words at 4, the step to 2 pays
+  // only below one CTA for two SMs: 6 inputs x 256 channels x 1024 spectra (192
+  // CTAs at 4) 15 us at 4 against 21 at 2 (29 with its pieces in bytes), 3 x 64 x
+  // 4096 with spectra (128) 11 against 12.8 (15); 16 x 64 x 200 (32) 10.9 against
+  // 9.0.  (Not for 16 and 32 channels, whose units are 4 and 8 threads: 16 x 16 x
+  // 4096 8.6 at 4 against 7.0.)
   FeArgs b = a;
+  const bool pieces = LOGM >= 7 && a.out && a.layout == CORR_L_CIT &&
+                      ((reinterpret_cast<uintptr_t>(a.out) | (uintptr_t)a.out_stride) & 3) == 0;
   const int slots = device_sm_count() * fe_min_blocks(LOGM);
   for (b.per_unit = 32; b.per_unit > 2; b.per_unit /= 2) {
     const int group = b.per_unit * fe_units(LOGM);
     const long long ctas = (long long)((a.n_spectra + group - 1) / group) * n_pairs;
     if (b.per_unit == 32 && ctas > slots && ctas < 2 * slots) continue;
-    if (ctas >= slots * 5 / 6) break;
+    if (ctas >= (pieces && b.per_unit == 4 ? device_sm_count() / 2 : slots * 5 / 6)) break;
   }
+  // (64 inputs x 64 channels x 128 spectra 10.6 us in bytes, 8.6 in half words)
+  b.vec_two = b.per_unit == 2 && ((reinterpret_cast<uintptr_t>(a.out) | (uintptr_t)a.out_stride) & 1) == 0;
   const int group = b.per_unit * fe_units(LOGM);
   // [t][c][i] codes: CTAs of neighbouring pairs, which write the same sectors, run
   // together, so that the L2 joins their bytes (192 inputs x 1024 channels x 2048
