@@ -72,6 +72,7 @@ __host__ __device__ constexpr int fe_units(int logm) { return fe_threads(logm) /
 // spectra, two spectra of both inputs to a word.  Only the thread itself reads
 // them back.
 constexpr int kStageIts = 8;
+constexpr long long kL2Bytes = 120 << 20;  // what the L2 holds of a kernel's output (126 MB)
 template <int LOGM>
 constexpr size_t fe_smem_bytes() {
   constexpr int M = 1 << LOGM;
@@ -806,6 +807,7 @@ __global__ void __launch_bounds__(fe_threads(LOGM), fe_min_blocks(LOGM)) fengine
 
 template <int LOGM, bool POWER, bool FRAMED, bool EXTRA>
 cudaError_t fe_launch_one(const FeArgs& a, int n_pairs, cudaStream_t s) {
+  constexpr int M = 1 << LOGM;
   constexpr size_t smem = fe_smem_bytes<LOGM>();
   static bool attr = false;
   if (!attr) {
@@ -841,13 +843,22 @@ cudaError_t fe_launch_one(const FeArgs& a, int n_pairs, cudaStream_t s) {
   // (64 inputs x 64 channels x 128 spectra 10.6 us in bytes, 8.6 in half words)
   b.vec_two = b.per_unit == 2 && ((reinterpret_cast<uintptr_t>(a.out) | (uintptr_t)a.out_stride) & 1) == 0;
   const int group = b.per_unit * fe_units(LOGM);
-  // [t][c][i] codes: CTAs of neighbouring pairs, which write the same sectors, run
-  // together, so that the L2 joins their bytes (192 inputs x 1024 channels x 2048
-  // spectra 5.5 -> 2.35 ms; the half-word stores alone 5.1, and 64 x 512 x 2048
-  // 480 -> 315 us).  The spectra and 18-bit values lie the same way (192 x 1024 x
-  // 512, one of them 1.37 -> 0.91 ms, and 0.63 with both inputs' as 16 bytes).
+  // [t][c][i] codes, spectra and 18-bit values: the inputs of a pair are 2 bytes of
+  // codes, 8 or 16 of the others, so neighbouring pairs write the same sectors.
+  // Together they may be larger than the L2, which then writes out sectors before
+  // their other pairs come: CTAs of neighbouring pairs run together (192 inputs x
+  // 1024 channels x 2048 spectra 5.1 -> 2.35 ms, 191 x 256 x 8192 5.55 -> 3.05;
+  // spectra of 64 x 1024 x 512 276 -> 210 us).  What fits joins there in any order,
+  // and neighbouring groups of spectra, which share frames, are better run
+  // together (191 x 1024 x 64 codes 167 -> 140 us, 33 x 64 x 2048 33.5 -> 31.2).
+  // The line lies between 113 MB, where groups are ahead by up to 17%, and 133 MB,
+  // where pairs are by 5 to 50%.  With spectra or 18-bit values groups are ahead
+  // below it only from many pairs on (191 x 256 x 128 and codes 121 -> 95 us; 17 and
+  // 33 inputs 3 to 14% the other way, 9 and 65 mixed).
   const int groups = (a.n_spectra + group - 1) / group;
-  b.pairs_first = ((a.out && a.layout != CORR_L_CIT) || a.spec || a.v18) && groups <= 65535;
+  const long long samples = (long long)M * a.n_spectra * n_pairs;  // (of both inputs: M / 2 channels)
+  const long long joined = samples * ((a.out && a.layout != CORR_L_CIT ? 1 : 0) + (a.spec ? 8 : 0) + (a.v18 ? 8 : 0));
+  b.pairs_first = (joined > kL2Bytes || ((a.spec || a.v18) && n_pairs <= 64)) && groups <= 65535;
   const dim3 grid = b.pairs_first ? dim3(n_pairs, groups) : dim3(groups, n_pairs);
   fengine_kernel<LOGM, POWER, FRAMED, EXTRA><<<grid, fe_threads(LOGM), smem, s>>>(b);
   return cudaGetLastError();
