@@ -196,7 +196,7 @@ std::vector<HerkTask> plan_tasks(int n_inputs, int n_chans, int* rows_per_chan, 
 // The same in 256 x 256 tasks for pairs of CTAs: {channel, super row, {super
 // column, -1}}.  pair_tasks_pay: whether an array is better multiplied so.
 std::vector<HerkTask> plan_pair_tasks(int n_inputs, int n_chans);
-bool pair_tasks_pay(int bits, int n_inputs);
+bool pair_tasks_pay(int bits, int n_inputs, int n_chans, int n_time);
 
 // Snapshot the device status word into host_slot (pinned host memory, written
 // by the device through its mapping; read it once the stream has passed this

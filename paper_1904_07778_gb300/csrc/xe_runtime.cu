@@ -132,7 +132,20 @@ std::vector<HerkTask> plan_pair_tasks(int n, int c) {
 // 448; from four on pairs move less.  Measured at 64 channels, push and dump:
 // 200 inputs (x 2048 spectra) 87 -> 78 us, 256 (128 channels, 4096) 217 -> 179,
 // 320 (1024) 68 -> 64, 448 (4096) 302 -> 272, 512 (4096) 391 -> 274.
-bool pair_tasks_pay(int bits, int n_inputs) { return bits == 8 && n_inputs > 192; }
+// Short blocks are bound by the drains, and with five row blocks (257 .. 320
+// inputs), half of the last super row empty, pairs drain more: up to 256 spectra
+// they are ahead only while the tasks do not fill the chip a few times over (257
+// inputs x 256 spectra x 16, 64, 200, 400 channels: 0.92, 0.99, 1.05, 1.09 of the
+// single CTAs' time; 320 inputs 0.85, 0.82, 0.98, 1.03).  With seven the same up
+// to 128 spectra (385 x 128 x 200, 400: 1.05, 1.08); with nine or more, or an even
+// count, pairs are ahead or equal at every length.
+bool pair_tasks_pay(int bits, int n_inputs, int n_chans, int n_time) {
+  if (bits != 8 || n_inputs <= 192) return false;
+  const int nrb = (2 * n_inputs + 127) / 128;
+  if (nrb == 5) return n_time > 256 || n_chans < 150;
+  if (nrb == 7) return n_time > 128 || n_chans < 200;
+  return true;
+}
 
 }  // namespace xe
 
@@ -556,7 +569,7 @@ int corr_create(int n_inputs, int n_chans, int n_time, int bits, int layout, uns
     }
     if (st != CORR_OK) break;
     std::vector<HerkTask> tasks = plan_tasks(n_inputs, n_chans, &x->rows_per_chan);
-    x->pair = pair_tasks_pay(bits, n_inputs);
+    x->pair = pair_tasks_pay(bits, n_inputs, n_chans, n_time);
     if (x->pair && turn_can_persist(layout, bits)) {
       x->n_single_tasks = (int)tasks.size();
       if (cudaMalloc(&x->single_tasks, tasks.size() * sizeof(HerkTask)) != cudaSuccess) { st = CORR_ENOMEM; break; }

@@ -199,7 +199,7 @@ void admit(corr_svc* s) {
     q.slot = s->free_slots.back();
     s->free_slots.pop_back();
     q.tasks = plan_tasks(q.r.n_inputs, q.r.n_chans, &q.rpc);
-    q.pair = pair_tasks_pay(q.r.bits, q.r.n_inputs);
+    q.pair = pair_tasks_pay(q.r.bits, q.r.n_inputs, q.r.n_chans, q.r.block_spectra);
     if (q.pair) q.tasks = plan_pair_tasks(q.r.n_inputs, q.r.n_chans);
     if (!s->dry) {
       for (int b = 0; b < 2; ++b) {

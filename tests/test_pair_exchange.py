@@ -53,3 +53,32 @@ def test_long_runs_of_pairs_repeat(N, C, T, layout):
     x = b.reshape((T, C, N, 2) if layout == 0 else (C, N, T, 2))
     one = np.ascontiguousarray(x[:, c] if layout == 0 else x[c])
     assert np.array_equal(vis[0][c:c + 1].cpu().numpy(), oracle.correlate(one, N, 1, T, bits=8, layout=layout))
+
+
+@pytest.mark.parametrize("N,C,T", [(257, 149, 256), (257, 150, 256), (257, 150, 257), (385, 200, 128), (385, 200, 129)])
+def test_pairs_or_single_ctas_by_size(N, C, T):
+    """On both sides of the lines between pairs and single CTAs: one context,
+    several blocks a launch, and the service."""
+    import torch
+    from paper_1904_07778_gb300 import xengine as xe
+    b = _block(N + C, 2 * N * C * T)
+    d = torch.from_numpy(b).cuda()
+    with xe.Correlator(N, C, T, bits=8, layout=xe.CORR_L_CIT) as cor:
+        cor.push(d)
+        vis = cor.dump()
+    x = b.reshape(C, N, T, 2)
+    for c in (0, C - 1):
+        one = np.ascontiguousarray(x[c])
+        assert np.array_equal(vis[c:c + 1], oracle.correlate(one, N, 1, T, bits=8, layout=xe.CORR_L_CIT))
+    tci = np.ascontiguousarray(x.transpose(2, 0, 1, 3))
+    dt = torch.from_numpy(tci).cuda().view(-1)
+    with xe.Correlator(N, C, T, bits=8, layout=xe.CORR_L_TCI) as cor:
+        cor.push_many([dt, dt])
+        assert np.array_equal(cor.dump(), 2 * vis)
+    with xe.Service(1 << 30) as svc:
+        rid = svc.submit(N, C, 8, xe.CORR_L_TCI, T, 1)
+        torch.cuda.synchronize()
+        svc.push(rid, dt)
+        svc.tick()
+        assert svc.wait() == xe.CORR_OK
+        assert np.array_equal(svc.fetch(rid), vis)
