@@ -72,7 +72,7 @@ __host__ __device__ constexpr int fe_units(int logm) { return fe_threads(logm) /
 // spectra, two spectra of both inputs to a word.  Only the thread itself reads
 // them back.
 constexpr int kStageIts = 8;
-constexpr long long kL2Bytes = 120 << 20;  // what the L2 holds of a kernel's output (126 MB)
+constexpr long long kL2Bytes = 120 << 20;  // what the L2 (135 MB) holds of a kernel's output
 template <int LOGM>
 constexpr size_t fe_smem_bytes() {
   constexpr int M = 1 << LOGM;
@@ -822,8 +822,9 @@ cudaError_t fe_launch_one(const FeArgs& a, int n_pairs, cudaStream_t s) {
   // 64 x 64 x 2048 33 us at 16 (256) against 39 at 4; 16 x 128 x 100 10.8 at 2
   // against 57 at 32.
   // (From 32 to 16, whose pieces are as large, also where 32 leave between one
-  // and two CTAs a slot: 32 x 256 x 4096 with powers, to visibilities, 174 us at
-  // 16 against 180 at 32, 512 CTAs.)
+  // and 16/9 CTAs a slot, for fuller waves: over 16 to 1024 channels and 8 to 192
+  // inputs, with powers and without, 16 take 0.83 - 0.90 of the time of 32 at 305
+  // to 368 CTAs, 0.97 - 1.03 to 448, 0.91 - 0.96 to 530, and 1.03 - 1.08 from 560 on.)
   // Where the pieces of [c][i][t] codes are whole words at 4, the step to 2 pays
   // only below one CTA for two SMs: 6 inputs x 256 channels x 1024 spectra (192
   // CTAs at 4) 15 us at 4 against 21 at 2 (29 with its pieces in bytes), 3 x 64 x
@@ -837,7 +838,7 @@ cudaError_t fe_launch_one(const FeArgs& a, int n_pairs, cudaStream_t s) {
   for (b.per_unit = 32; b.per_unit > 2; b.per_unit /= 2) {
     const int group = b.per_unit * fe_units(LOGM);
     const long long ctas = (long long)((a.n_spectra + group - 1) / group) * n_pairs;
-    if (b.per_unit == 32 && ctas > slots && ctas < 2 * slots) continue;
+    if (b.per_unit == 32 && ctas > slots && ctas <= slots * 16 / 9) continue;
     if (ctas >= (pieces && b.per_unit == 4 ? device_sm_count() / 2 : slots * 5 / 6)) break;
   }
   // (64 inputs x 64 channels x 128 spectra 10.6 us in bytes, 8.6 in half words)
