@@ -442,9 +442,8 @@ __global__ void pad_rows_kernel(const uint8_t* __restrict__ in, uint8_t* __restr
 // D - s^2 and a - q s are then below 2^63 and exact in the low 64 bits of
 // integer products; they give the correction to within half a unit and a
 // little, and the new remainder's sign against half a unit the last step.  So
-// the results are those of sqrt and / (also compared over 10^9 random
-// operands, without a difference).  One FP64 product a baseline is left, the
-// denominator's square.  What bounds it now is the issue of some 230
+// the results are those of sqrt and /.  One FP64 product a baseline is left,
+// the denominator's square.  What bounds it now is the issue of some 230
 // instructions a baseline (74% of the slots), then the 32 bytes (0.09 ms).
 // The call (192 inputs x 1024 channels): 163 us; 345 with the roundings by
 // FP64 residuals (7 operations of that pipe), 471 with the estimates in FP64
