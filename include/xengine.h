@@ -572,10 +572,6 @@ int corr_svc_state(corr_svc* s, int64_t id, int* state);
  * CORR_EBUSY while two pushed blocks are waiting for ticks. */
 int corr_svc_push(corr_svc* s, int64_t id, const void* block, size_t nbytes);
 
-/* The cudaStream_t of the copies that corr_svc_push queues, for ordering other
- * work with them.  NULL for a null service or a dry run. */
-void* corr_svc_ingest_stream(corr_svc* s);
-
 /* corr_svc_tick -- correlate the oldest waiting block of every active
  * request in one launch per sample width.  *n_requests (optional) receives
  * how many requests took part.  Asynchronous. */

@@ -348,8 +348,6 @@ int corr_svc_push(corr_svc* s, int64_t id, const void* block, size_t nbytes) {
   return CORR_OK;
 }
 
-void* corr_svc_ingest_stream(corr_svc* s) { return s ? (void*)s->copy_stream : nullptr; }
-
 int corr_svc_tick(corr_svc* s, int* n_requests) {
   TraceRange trace_("corr_svc_tick");
   if (!s) return CORR_EINVAL;

@@ -186,25 +186,23 @@ def _ptr_and_size(buf):
 class _CopyStream:
     """Copies out of torch tensors on a stream of the library's: each waits for
     what torch's current stream has queued (the tensor's producer, usually),
-    and the tensor lives until its copy is done.  ``unordered``: a stream whose
-    work the copies do not wait for.  No handle: nothing is copied."""
+    and the tensor lives until its copy is done."""
 
-    def __init__(self, handle, unordered=None):
+    def __init__(self, handle):
         self._handle, self._stream, self._busy = handle, None, collections.deque()
-        self._unordered = (handle, unordered)
 
     def before(self, src):
-        if not self._handle or not getattr(src, "is_cuda", False):
+        if not getattr(src, "is_cuda", False):
             return
         import torch
         if self._stream is None:
             self._stream = torch.cuda.ExternalStream(self._handle)
         cur = torch.cuda.current_stream()
-        if cur.cuda_stream not in self._unordered and not torch.cuda.is_current_stream_capturing():
+        if cur.cuda_stream != self._handle and not torch.cuda.is_current_stream_capturing():
             self._stream.wait_stream(cur)
 
     def after(self, src):
-        if not self._handle or not hasattr(src, "data_ptr"):
+        if not hasattr(src, "data_ptr"):
             return
         import torch
         if not torch.cuda.is_available():
@@ -541,8 +539,7 @@ class Batch:
 
 # ------------------------------------------------------------------- service
 EXPORTS += ["corr_svc_create", "corr_svc_submit", "corr_svc_state", "corr_svc_push", "corr_svc_tick",
-            "corr_svc_fetch", "corr_svc_wait", "corr_svc_stats_get", "corr_svc_destroy",
-            "corr_svc_ingest_stream"]
+            "corr_svc_fetch", "corr_svc_wait", "corr_svc_stats_get", "corr_svc_destroy"]
 CORR_SVC_DRY_RUN = 1
 CORR_REQ_QUEUED, CORR_REQ_ACTIVE, CORR_REQ_DONE, CORR_REQ_FETCHED = 0, 1, 2, 3
 
@@ -572,8 +569,6 @@ _lib.corr_svc_push.argtypes = [_P, ctypes.c_int64, _P, _SZ]
 _lib.corr_svc_tick.argtypes = [_P, ctypes.POINTER(_I)]
 _lib.corr_svc_fetch.argtypes = [_P, ctypes.c_int64, _P]
 _lib.corr_svc_wait.argtypes = [_P]
-_lib.corr_svc_ingest_stream.argtypes = [_P]
-_lib.corr_svc_ingest_stream.restype = _P
 _lib.corr_svc_stats_get.argtypes = [_P, ctypes.POINTER(CorrSvcStats)]
 _lib.corr_svc_destroy.argtypes = [_P]
 _lib.corr_svc_destroy.restype = None
@@ -595,8 +590,6 @@ class Service:
         if st != CORR_OK:
             raise CorrError(st, "corr_svc_create")
         self._s = out
-        # (a copy that waited for the ticks' own stream would not overlap them)
-        self._copies = _CopyStream(_lib.corr_svc_ingest_stream(out), stream)
         self._shape = {}
 
     def submit(self, n_inputs, n_chans, bits, layout, block_spectra, n_blocks, flags=0, check=True):
@@ -618,16 +611,9 @@ class Service:
         return out.value
 
     def push(self, rid, block, check=True):
-        """Queue the copy of the request's next block.  A torch tensor is kept
-        until it is copied, and its copy follows the work queued on torch's
-        current stream; on the stream that the service was made for, the tensor
-        has to be complete (corr_svc_push)."""
         p, n = _ptr_and_size(block)
-        self._copies.before(block)
         st = _lib.corr_svc_push(self._s, rid, _P(p), n)
-        if st == CORR_OK:
-            self._copies.after(block)
-        elif check:
+        if check and st != CORR_OK:
             raise CorrError(st, "corr_svc_push")
         return st
 
@@ -652,9 +638,7 @@ class Service:
         return vis
 
     def wait(self):
-        st = _lib.corr_svc_wait(self._s)
-        self._copies.synchronised()
-        return st
+        return _lib.corr_svc_wait(self._s)
 
     def stats(self):
         out = CorrSvcStats()
@@ -667,7 +651,6 @@ class Service:
         if getattr(self, "_s", None):
             _lib.corr_svc_destroy(self._s)
             self._s = None
-            self._copies.synchronised()
 
     def __enter__(self):
         return self

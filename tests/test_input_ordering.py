@@ -55,66 +55,3 @@ def test_batch_input_lives_until_it_is_copied():
         b.run()
         assert b.sync() == xe.CORR_OK
         assert np.array_equal(b.output(0), oracle.correlate(blk, *SHAPE[:3], layout=0))
-
-
-@pytest.mark.parametrize("side_stream", [False, True])
-def test_service_block_follows_its_producer(side_stream):
-    from paper_1904_07778_gb300 import xengine as xe
-    n, c, t, bits, layout = SHAPE
-    blk = _samples(3)
-    src = torch.from_numpy(blk).cuda()
-    dst = torch.zeros_like(src)
-    torch.cuda.synchronize()
-    with xe.Service(1 << 28) as svc:
-        rid = svc.submit(n, c, bits, layout, t, 1)
-        st = torch.cuda.Stream() if side_stream else torch.cuda.current_stream()
-        with torch.cuda.stream(st):
-            torch.cuda._sleep(40_000_000)
-            dst.copy_(src)
-            svc.push(rid, dst)
-        svc.tick()
-        assert svc.wait() == xe.CORR_OK
-        assert np.array_equal(svc.fetch(rid), oracle.correlate(blk, n, c, t, layout=layout))
-
-
-def test_service_block_lives_until_it_is_copied():
-    from paper_1904_07778_gb300 import xengine as xe
-    n, c, t, bits, layout = SHAPE
-    blk = _samples(4)
-    with xe.Service(1 << 30) as svc:
-        first = svc.submit(192, 256, 4, 0, 4096, 1)       # its copy goes before the block's
-        rid = svc.submit(n, c, bits, layout, t, 1)
-        big = torch.zeros(192 * 256 * 4096, dtype=torch.uint8, device="cuda")
-        b = torch.from_numpy(blk).cuda()
-        torch.cuda.synchronize()
-        at = b.data_ptr()
-        svc.push(first, big)
-        svc.push(rid, b)
-        del b
-        other = [torch.full((BYTES,), 0x77, dtype=torch.uint8, device="cuda") for _ in range(4)]
-        assert at not in [o.data_ptr() for o in other]
-        svc.tick()
-        assert svc.wait() == xe.CORR_OK
-        assert np.array_equal(svc.fetch(rid), oracle.correlate(blk, n, c, t, layout=layout))
-
-
-def test_held_blocks_are_let_go():
-    """Neither the batch nor the service keeps a tensor past the next
-    synchronisation, nor more of them than are in flight."""
-    import gc
-    import weakref
-    from paper_1904_07778_gb300 import xengine as xe
-    n, c, t, bits, layout = SHAPE
-    with xe.Batch([SHAPE]) as batch, xe.Service(1 << 28) as svc:
-        x = torch.from_numpy(_samples(5)).cuda()
-        y = torch.from_numpy(_samples(6)).cuda()
-        torch.cuda.synchronize()
-        refs = [weakref.ref(x), weakref.ref(y)]
-        batch.set_input(0, x)
-        svc.push(svc.submit(n, c, bits, layout, t, 1), y)
-        del x, y
-        batch.sync()
-        svc.tick()
-        svc.wait()
-        gc.collect()
-        assert [r() for r in refs] == [None, None]
