@@ -189,33 +189,36 @@ class _CopyStream:
     and the tensor lives until its copy is done."""
 
     def __init__(self, handle):
-        self._handle, self._stream, self._busy = handle, None, collections.deque()
+        self._handle, self._stream, self._produced = handle, None, None
+        self._busy, self._spare = collections.deque(), []
+
+    def _torch(self):
+        import torch
+        if self._stream is None:
+            self._stream, self._produced = torch.cuda.ExternalStream(self._handle), torch.cuda.Event()
+        return torch
 
     def before(self, src):
         if not getattr(src, "is_cuda", False):
             return
-        import torch
-        if self._stream is None:
-            self._stream = torch.cuda.ExternalStream(self._handle)
+        torch = self._torch()
         cur = torch.cuda.current_stream()
         if cur.cuda_stream != self._handle and not torch.cuda.is_current_stream_capturing():
-            self._stream.wait_stream(cur)
+            self._produced.record(cur)          # (the wait takes the record of now)
+            self._stream.wait_event(self._produced)
 
     def after(self, src):
         if not hasattr(src, "data_ptr"):
             return
-        import torch
-        if not torch.cuda.is_available():
-            return
-        if self._stream is None:
-            self._stream = torch.cuda.ExternalStream(self._handle)
+        torch = self._torch()
         while self._busy and self._busy[0][0].query():
-            self._busy.popleft()
-        done = torch.cuda.Event()
+            self._spare.append(self._busy.popleft()[0])
+        done = self._spare.pop() if self._spare else torch.cuda.Event()
         done.record(self._stream)
         self._busy.append((done, src))
 
     def synchronised(self):
+        self._spare.extend(done for done, _ in self._busy)
         self._busy.clear()
 
 
@@ -611,6 +614,11 @@ class Service:
         return out.value
 
     def push(self, rid, block, check=True):
+        """Queue the copy of the request's next block on the ingest stream.  A
+        device block has to be complete (synchronise its producer first) and to
+        be kept, unchanged, until :meth:`wait` or the end of the tick that
+        integrates it: the copy is ordered after nothing, and nothing here holds
+        the tensor."""
         p, n = _ptr_and_size(block)
         st = _lib.corr_svc_push(self._s, rid, _P(p), n)
         if check and st != CORR_OK:

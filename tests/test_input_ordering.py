@@ -55,3 +55,24 @@ def test_batch_input_lives_until_it_is_copied():
         b.run()
         assert b.sync() == xe.CORR_OK
         assert np.array_equal(b.output(0), oracle.correlate(blk, *SHAPE[:3], layout=0))
+
+
+def test_held_inputs_are_let_go():
+    """The batch keeps no tensor past the next synchronisation, nor more of
+    them than are in flight."""
+    import gc
+    import weakref
+    from paper_1904_07778_gb300 import xengine as xe
+    with xe.Batch([SHAPE]) as b:
+        refs = []
+        for k in range(3):
+            x = torch.from_numpy(_samples(5 + k)).cuda()
+            refs.append(weakref.ref(x))
+            b.set_input(0, x)
+            torch.cuda.synchronize()
+        del x
+        gc.collect()
+        assert [r() is None for r in refs] == [True, True, False]   # each call lets earlier ones go
+        b.sync()
+        gc.collect()
+        assert refs[2]() is None
