@@ -184,9 +184,9 @@ def _ptr_and_size(buf):
 
 
 class _CopyStream:
-    """Copies out of torch tensors on a stream of the library's: each waits for
-    what torch's current stream has queued (the tensor's producer, usually),
-    and the tensor lives until its copy is done."""
+    """Copies out of torch tensors on a stream of the library's: ``follow``
+    orders them after the work queued on a torch stream, and ``hold`` keeps a
+    tensor until its copy is done."""
 
     def __init__(self, handle):
         self._handle, self._stream, self._produced = handle, None, None
@@ -198,18 +198,13 @@ class _CopyStream:
             self._stream, self._produced = torch.cuda.ExternalStream(self._handle), torch.cuda.Event()
         return torch
 
-    def before(self, src):
-        if not getattr(src, "is_cuda", False):
-            return
-        torch = self._torch()
-        cur = torch.cuda.current_stream()
-        if cur.cuda_stream != self._handle and not torch.cuda.is_current_stream_capturing():
-            self._produced.record(cur)          # (the wait takes the record of now)
+    def follow(self, producer):
+        self._torch()
+        if producer.cuda_stream != self._handle:
+            self._produced.record(producer)     # (the wait takes the record of now)
             self._stream.wait_event(self._produced)
 
-    def after(self, src):
-        if not hasattr(src, "data_ptr"):
-            return
+    def hold(self, src):
         torch = self._torch()
         while self._busy and self._busy[0][0].query():
             self._spare.append(self._busy.popleft()[0])
@@ -471,17 +466,22 @@ class Batch:
         self._b = out
         self._copies = _CopyStream(_lib.corr_batch_stream(out))
 
-    def set_input(self, k, block):
-        """Queue the copy of ``block`` (host or device) into array k's input.
-        A torch tensor's copy follows the work queued on torch's current
-        stream, and the tensor is kept until it is done; its contents may be
-        changed after :meth:`sync`."""
+    def set_input(self, k, block, after=None):
+        """Queue the copy of ``block`` (host or device) into array k's input, on
+        the batch's stream.  ``after``: a torch stream whose queued work the copy
+        follows, for a tensor that it is still writing.  Without it the block has
+        to be complete at the call, as for corr_batch_set_input: a batch made on
+        torch's default stream runs on a stream of its own, which waits for no
+        other.  A torch tensor is kept until its copy is done; its contents may
+        be changed after :meth:`sync`."""
         p, n = _ptr_and_size(block)
-        self._copies.before(block)
+        if after is not None:
+            self._copies.follow(after)
         st = _lib.corr_batch_set_input(self._b, k, _P(p), n)
         if st != CORR_OK:
             raise CorrError(st, "corr_batch_set_input")
-        self._copies.after(block)
+        if hasattr(block, "data_ptr"):
+            self._copies.hold(block)
 
     def output(self, k):
         n, c = self.shapes[k][0], self.shapes[k][1]

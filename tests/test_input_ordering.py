@@ -1,6 +1,6 @@
 """Device tensors handed over for a copy on a stream of the library's own: the
-copy follows the work queued on torch's current stream, and the tensor's
-memory is not given to another before the copy is done."""
+copy follows the work queued on the stream that the caller names, and the
+tensor's memory is not given to another before the copy is done."""
 import numpy as np
 import pytest
 
@@ -31,7 +31,7 @@ def test_batch_input_follows_its_producer(side_stream):
         with torch.cuda.stream(st):
             torch.cuda._sleep(40_000_000)   # the producer is late (about 20 ms)
             dst.copy_(src)
-            b.set_input(0, dst)
+            b.set_input(0, dst, after=torch.cuda.current_stream())
         b.run()
         assert b.sync() == xe.CORR_OK
         assert np.array_equal(b.output(0), oracle.correlate(blk, *SHAPE[:3], layout=0))
