@@ -402,7 +402,7 @@ __host__ __device__ constexpr int fe_min_blocks(int logm) { return logm <= 11 ? 
 
 // What bounds it: latency.  128 registers a thread (32 hold the two spectra's
 // eight points, 52 the taps and the next frames) leave 16 warps an SM, with
-// issue slots half busy, the shared-memory data pipe 58% and FP32 42%; the time
+// issue slots 47% busy, the shared-memory data pipe 62% and FP32 42%; the time
 // is close to proportional to the instructions of an iteration (about 1250 a
 // thread), a quarter of them the separation and equaliser.  192 inputs x 1024
 // channels x 2048 spectra: 2.02 -> 1.50 ms, in steps (ms): packed pairs and
